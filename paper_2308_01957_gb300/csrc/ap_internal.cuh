@@ -65,21 +65,30 @@ struct SourceDev {
   int64_t j_off;     // element offset of this source's convolved columns (-1: none)
 };
 
-// Per-evaluation source record, prepared from theta on the device.
+// Per-evaluation source record, prepared from theta on the device.  A profile
+// (Sersic ... Moffat) works in coordinates scaled by its radius R (Re, sigma,
+// Rd): x = X / R, y = Y / (q R), u = x^2 + y^2, so that a quadrature node
+// costs two FMAs for (x, y) and two for u, and every constant of the
+// derivatives is folded into one coefficient per sum (float64, once per
+// source; see pixel_derivs in ap_render.cu).
 template <typename T>
 struct SrcPar {
-  T m00, m01, m10, m11;  // X = m00 du + m01 dv, Y = m10 du + m11 dv (du, dv pixel offsets);
-                         // sky plane: the pixel -> world matrix A
-  T invq;
+  T m00, m01, m10, m11;  // x = m00 du + m01 dv, y = m10 du + m11 dv (du, dv pixel offsets);
+                         // sky plane: the pixel -> world matrix A; PSF star: A^-1
   T fx, fy;              // centre's fractional position in its reference pixel; sky plane:
                          // the image centre in pixels (W/2, H/2)
   T area;
-  T c, s;                // cos PA, sin PA
-  T k0, k1, k2, k3, k4, k5, k6;  // profile constants (see ap_render.cu)
-  T pv[MAX_SLOTS];       // slot values
+  T amp;                 // value scale: area Ie, area F norm
+  T k0, k1, k2;          // Sersic: 1/(2n), softening of u, b log2(e); Gaussian: -log2(e)/2;
+                         // Moffat: n; sky: the slot values; PSF star: F, map centre
+  // derivative coefficients: D0 = c0x Sx + c0y Sy, D1 = c1x Sx + c1y Sy,
+  // D2 = c2 Syy + c2s S1, D3 = c3 Sxy, then c4a, c4b, c5a, c5b, c6 by type
+  T c0x, c0y, c1x, c1y, c2, c2s, c3, c4a, c4b, c5a, c5b, c6;
+  T pad0_;
   int jc, ic;            // reference pixel (column, row)
   int pad_[2];
 };
+static_assert(sizeof(SrcPar<float>) % 16 == 0 && sizeof(SrcPar<double>) % 16 == 0, "records of whole 16-byte words");
 
 // Work items.
 struct TileWork {        // one TILE x TILE tile of a layer
