@@ -52,7 +52,6 @@ struct ap_ctx {
   int* d_fwd_valid = nullptr;            // per group: current records / w r / chi2_state in place
   StateChunk* d_state_chunks = nullptr;  // trial -> current copies of an accepted group
   int n_state_chunks = 0;
-  double* d_bn_memo = nullptr;   // per source: the last two (n, b_n, db/dn) of prepare_kernel
   // render / adjoint-render plan
   TileWork* d_rwork = nullptr;
   int n_rwork = 0;
@@ -313,7 +312,7 @@ int do_eval(ap_ctx* c, const double* theta, double* chi2_out, double* grad_out, 
                           (grad_out ? (c->n_awork > 0) + (c->n_rwork > 0) + (c->n_params > 0) : 0);
   {
     Bracket b(c, st, "prepare");
-    launch_prepare<T>(c->d_srcs, c->d_imgs, c->n_src, theta, par, c->d_bn_memo, skip, c->d_status, st);
+    launch_prepare<T>(c->d_srcs, c->d_imgs, c->n_src, theta, par, skip, c->d_status, st);
   }
   if (c->n_live > 0) {
     // every evaluation renders the live PSFs at its theta (never skipped: the
@@ -564,7 +563,7 @@ void eval_shifted(ap_ctx* c, const double* theta, int method, double* chi2_out, 
   SrcPar<T>* par = (SrcPar<T>*)c->d_par;
   {
     Bracket b(c, st, "prepare");
-    launch_prepare<T>(c->d_srcs, c->d_imgs, c->n_src, theta, par, c->d_bn_memo, nullptr, c->d_status, st);
+    launch_prepare<T>(c->d_srcs, c->d_imgs, c->n_src, theta, par, nullptr, c->d_status, st);
   }
   if (c->n_live > 0) {
     Bracket b(c, st, "live_psf");
@@ -593,7 +592,7 @@ void eval_adaptive(ap_ctx* c, const double* theta, double tol, double* chi2_out,
   SrcPar<T>* par = (SrcPar<T>*)c->d_par;
   {
     Bracket b(c, st, "prepare");
-    launch_prepare<T>(c->d_srcs, c->d_imgs, c->n_src, theta, par, c->d_bn_memo, nullptr, c->d_status, st);
+    launch_prepare<T>(c->d_srcs, c->d_imgs, c->n_src, theta, par, nullptr, c->d_status, st);
   }
   if (c->n_live > 0) {
     Bracket b(c, st, "live_psf");
@@ -1580,8 +1579,6 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
     c->max_live_tiles = std::max(c->max_live_tiles, ((I[i].H + 15) / 16) * ((I[i].W + 15) / 16));
   if ((rc = upload(c, &c->d_imgs, I))) return rc;
   if ((rc = upload(c, &c->d_srcs, S))) return rc;
-  if ((rc = dev_alloc(c, (void**)&c->d_bn_memo, (size_t)std::max(n_src, 1) * 8 * sizeof(double)))) return rc;
-  CUDA_TRY(c, cudaMemset(c->d_bn_memo, 0xff, (size_t)std::max(n_src, 1) * 8 * sizeof(double)));   // NaN: no entry
   const size_t par_bytes = f64 ? sizeof(SrcPar<double>) : sizeof(SrcPar<float>);
   if ((rc = dev_alloc(c, &c->d_par, (size_t)std::max(n_src, 1) * par_bytes))) return rc;
   if ((rc = dev_alloc(c, &c->d_par_trial, (size_t)std::max(n_src, 1) * par_bytes))) return rc;

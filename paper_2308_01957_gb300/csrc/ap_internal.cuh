@@ -117,7 +117,7 @@ struct JcolFftWork {     // one FFT block of one free slot of one source's Jacob
 // ---------------------------------------------------------------------------
 // launchers (each TU owns its kernels; T = float or double)
 // ---------------------------------------------------------------------------
-void upload_gl_rule(int Q);  // Gauss-Legendre nodes/weights to constant memory
+void upload_gl_rule(int Q);  // Gauss-Legendre nodes/weights and the b_n table to device memory
 
 // Let a kernel use as much dynamic shared memory as the device allows next to
 // its static shared memory (the opt-in is a cap; every launch asks for what
@@ -141,11 +141,9 @@ inline int allow_max_dynamic_smem(F* func) {
 // copies the group's kept value instead).  The LM iteration sets the flags
 // once its current point's records and w r are in place.
 
-// bn_memo: 8 doubles per source (two (n, b_n, db/dn) entries and the slot to
-// replace next), filled with NaN bytes when the problem is set
 template <typename T>
 void launch_prepare(const SourceDev* srcs, const ImageDev* imgs, int n_src, const double* theta,
-                    SrcPar<T>* par, double* bn_memo, const int* skip, int* status, cudaStream_t st);
+                    SrcPar<T>* par, const int* skip, int* status, cudaStream_t st);
 
 template <typename T>
 void launch_render(int Q, const TileWork* work, int n_work, const int* tile_src, const SourceDev* srcs,

@@ -58,9 +58,12 @@ static void legendre_rule(int Q, double* x, double* w) {
   }
 }
 
+static void build_bn_table();
+
 void upload_gl_rule(int /*Q*/) {
   static bool done = false;
   if (done) return;
+  build_bn_table();
   float hu_f[8][8] = {}, hw_f[8][8] = {};
   double hu_d[8][8] = {}, hw_d[8][8] = {};
   for (int Q = 1; Q <= 7; ++Q) {
@@ -117,125 +120,168 @@ constexpr double LOG2E = 1.4426950408889634074;
 constexpr double LN2 = 0.69314718055994530942;
 
 // ---------------------------------------------------------------------------
-// Sersic b_n in float64 (Sersic 1963; half the light inside Re):
-// root of P(2n, b) = 1/2 with P the regularised lower incomplete gamma.
+// Sersic b_n (Sersic 1963; half the light inside Re): root of P(2n, b) = 1/2
+// with P the regularised lower incomplete gamma, and db/dn.  Both are smooth
+// functions of n alone, so the host tabulates them once per process as
+// piecewise polynomials (quarter octaves of n from 0.05 to 20, degree BN_DEG
+// through the Chebyshev points of each piece: the interpolation error is below
+// float64 rounding: 2e-16 of b_n against 40-digit roots) and the device
+// evaluates two Horner chains.  Solving for the root on the device took a warp
+// about 20 us of float64 latency at every new n.
 //  * P(a, x) by its power series x^a e^-x / Gamma(a+1) sum_k x^k / prod_{j<=k}(a+j)
 //    (the root satisfies x < a + 1, where the series converges geometrically);
 //  * dP/da by differentiating the series term by term, with the digamma
 //    function from its recurrence and asymptotic (Bernoulli) expansion;
-//  * safeguarded Newton from the Ciotti & Bertin (1999) asymptotic start,
-//    inside the bracket [0, a + 2];
+//  * Halley steps from the Ciotti & Bertin (1999) asymptotic start inside the
+//    bracket [0, a + 2], bisection when a step leaves it;
 //  * db/dn = -2 (dP/da) / (dP/dx), dP/dx = x^(a-1) e^-x / Gamma(a).
 // ---------------------------------------------------------------------------
-__device__ double digamma_pos(double z) {
-  double acc = 0.0;
-  while (z < 10.0) {
-    acc -= 1.0 / z;
-    z += 1.0;
+constexpr int BN_DEG = 14, BN_PIECES = 35;       // 8.65 octaves
+constexpr double BN_MIN = 0.05, BN_MAX = 20.0;   // n past these is refused
+struct BnPiece {
+  double mid, inv_half;                          // piece coordinate (n - mid) inv_half in [-1, 1]
+  double b[BN_DEG + 1], db[BN_DEG + 1];          // power coefficients, highest first
+};
+__device__ BnPiece c_bn[BN_PIECES];
+
+static long double digamma_ld(long double z) {
+  long double acc = 0.0L;
+  while (z < 20.0L) {
+    acc -= 1.0L / z;
+    z += 1.0L;
   }
-  double iz = 1.0 / z, iz2 = iz * iz;
-  double series = iz2 * (1.0 / 12.0 - iz2 * (1.0 / 120.0 - iz2 * (1.0 / 252.0 - iz2 * (1.0 / 240.0 - iz2 * (1.0 / 132.0)))));
-  return acc + log(z) - 0.5 * iz - series;
+  const long double r = 1.0L / (z * z);
+  const long double s = r * (1.0L / 12 - r * (1.0L / 120 - r * (1.0L / 252 - r * (1.0L / 240 - r * (1.0L / 132 -
+                        r * (691.0L / 32760 - r * (1.0L / 12)))))));
+  return acc + std::log(z) - 0.5L / z - s;
 }
 
-// Reciprocal in float64 by two Newton-Raphson steps r <- r (2 - d r) from a
-// float32 seed (relative error squares each step: 1e-7 -> 1e-14 -> 1e-28).
-__device__ __forceinline__ double recip64(double d) {
-  double r = (double)(1.0f / (float)d);
-  r = r * fma(-d, r, 2.0);
-  r = r * fma(-d, r, 2.0);
-  return r;
-}
-
-// One warp sums the series S = sum_{k>=0} x^k / prod_{j<=k}(a+j) and its
-// a-derivative dS = -sum_k t_k H_k, H_k = sum_{j<=k} 1/(a+j).  Lane l holds
-// the factor x/(a+k) of term k = 32c + l + 1; an inclusive multiplicative
-// shuffle scan gives a chunk of 32 terms, an additive scan the harmonic sums;
-// chunks continue from the previous chunk's last lane until a term drops
-// below 1e-18 (S >= 1).  Every lane returns the totals.
-__device__ void gamma_series_warp(double a, double x, double* S, double* dS) {
-  const int lane = threadIdx.x & 31;
-  double sum = 0.0, dsum = 0.0, carry_t = 1.0, carry_h = 0.0;
-  for (int chunk = 0; chunk < 8; ++chunk) {
-    const double ak = recip64(a + (double)(32 * chunk + lane + 1));
-    double t = x * ak, hs = ak;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const double tv = __shfl_up_sync(0xffffffffu, t, o);
-      const double hv = __shfl_up_sync(0xffffffffu, hs, o);
-      if (lane >= o) { t *= tv; hs += hv; }
+// b_n and db/dn at one n, in long double
+static void sersic_bn_ld(long double n, long double* b_out, long double* db_out) {
+  const long double a = 2.0L * n, lga = std::lgamma(a);
+  long double lo = 0.0L, hi = a + 2.0L;
+  long double b = a - 1.0L / 3 + 4.0L / (405 * n) + 46.0L / (25515 * n * n);
+  if (!(b > lo && b < hi) || n < 0.3L) b = std::exp((std::lgamma(a + 1.0L) - std::log(2.0L)) / a);   // small a: x^a / Gamma(a+1) = 1/2
+  long double fp = 0.0L, S = 1.0L, dS = 0.0L;
+  auto series = [&]() {
+    fp = std::exp((a - 1.0L) * std::log(b) - b - lga);
+    S = 1.0L;
+    dS = 0.0L;
+    long double t = 1.0L, h = 0.0L;
+    for (int k = 1; k < 400; ++k) {
+      const long double ak = 1.0L / (a + k);
+      t *= b * ak;
+      h += ak;
+      S += t;
+      dS -= t * h;
+      if (t < 1e-20L) break;
     }
-    t *= carry_t;
-    hs += carry_h;
-    sum += t;
-    dsum -= t * hs;
-    carry_t = __shfl_sync(0xffffffffu, t, 31);
-    carry_h = __shfl_sync(0xffffffffu, hs, 31);
-    if (carry_t < 1e-18) break;   // uniform: every lane holds the same carry
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
-  }
-  *S = 1.0 + sum;
-  *dS = dsum;
-}
-
-// All 32 lanes of a warp call this with the same n and get the same result.
-// With f'(b) = b^(a-1) e^-b / Gamma(a), P(a, b) = (b / a) f'(b) S(a, b), so an
-// iteration costs one exp, one log and one warp series.  Halley steps
-// (f''/f' = (a-1)/b - 1) inside the bracket [0, a + 2], bisection if a step
-// leaves it.
-__device__ void sersic_bn(double n, double* b_out, double* db_out, int* ok) {
-  const double a = 2.0 * n;
-  const double lga = lgamma(a);
-  double lo = 0.0, hi = a + 2.0;
-  double b = 2.0 * n - 1.0 / 3.0 + 4.0 / (405.0 * n) + 46.0 / (25515.0 * n * n);
-  if (!(b > lo && b < hi)) b = 0.5 * (lo + hi);
-  int conv = 0;
-  double fp = 0.0, S = 1.0, dS = 0.0;
+  };
   for (int it = 0; it < 60; ++it) {
-    fp = exp((a - 1.0) * log(b) - b - lga);
-    gamma_series_warp(a, b, &S, &dS);
-    const double f = b * fp * S / a - 0.5;
-    if (f < 0.0) lo = b; else hi = b;
-    const double h = f / fp;
-    const double c = (a - 1.0) / b - 1.0;
-    const double step = h / (1.0 - 0.5 * h * c);
-    // Halley converges cubically: once a step is below 1e-9 b the stepped
-    // iterate is accurate to float64 rounding.  (Tested before the bracket:
-    // a last step smaller than half an ulp lands on the bracket end.)
-    if (fabs(step) <= 1e-9 * b) { b -= step; conv = 1; break; }
-    double nb = b - step;
-    if (!(nb > lo && nb < hi)) nb = 0.5 * (lo + hi);
-    b = nb;
-    if (hi - lo <= 4e-16 * b) { conv = 1; break; }
+    series();
+    const long double f = b * fp * S / a - 0.5L;
+    (f < 0.0L ? lo : hi) = b;
+    const long double h = f / fp, c = (a - 1.0L) / b - 1.0L;
+    const long double step = h / (1.0L - 0.5L * h * c);
+    if (std::fabs(step) <= 1e-9L * b) {   // cubic convergence: the stepped iterate is accurate
+      b -= step;
+      break;
+    }
+    const long double nb = b - step;
+    b = nb > lo && nb < hi ? nb : 0.5L * (lo + hi);
   }
-  fp = exp((a - 1.0) * log(b) - b - lga);
-  gamma_series_warp(a, b, &S, &dS);
-  const double P = b * fp * S / a;
-  const double dPda = P * (log(b) - digamma_pos(a + 1.0)) + b * fp / a * dS;
+  series();
+  const long double P = b * fp * S / a;
   *b_out = b;
-  *db_out = -2.0 * dPda / fp;
-  *ok = conv && isfinite(b) && isfinite(*db_out);
+  *db_out = -2.0L * (P * (std::log(b) - digamma_ld(a + 1.0L)) + b * fp / a * dS) / fp;
+}
+
+static void build_bn_table() {
+  constexpr int M = BN_DEG + 1;
+  static BnPiece tab[BN_PIECES];
+  const long double pi = 3.14159265358979323846264338327950288L;
+  for (int p = 0; p < BN_PIECES; ++p) {
+    const long double n0 = BN_MIN * std::exp2(0.25L * p), n1 = n0 * std::exp2(0.25L);
+    const long double mid = 0.5L * (n0 + n1), half = 0.5L * (n1 - n0);
+    tab[p].mid = (double)mid;
+    tab[p].inv_half = (double)(1.0L / half);
+    long double f[2][M], c[2][M];
+    for (int k = 0; k < M; ++k) {
+      // the node in the device's own piece coordinate
+      const long double x = std::cos(pi * (k + 0.5L) / M);
+      sersic_bn_ld((long double)tab[p].mid + x / (long double)tab[p].inv_half, &f[0][k], &f[1][k]);
+    }
+    for (int q = 0; q < 2; ++q)
+      for (int j = 0; j < M; ++j) {
+        long double s = 0.0L;
+        for (int k = 0; k < M; ++k) s += f[q][k] * std::cos(pi * j * (k + 0.5L) / M);
+        c[q][j] = s * (j ? 2.0L : 1.0L) / M;
+      }
+    // Chebyshev to power coefficients: T_{j+1} = 2 x T_j - T_{j-1}
+    long double pw[2][M] = {}, t0[M] = {}, t1[M] = {};
+    t0[0] = 1.0L;
+    t1[1] = 1.0L;
+    for (int j = 0; j < M; ++j) {
+      for (int q = 0; q < 2; ++q)
+        for (int k = 0; k < M; ++k) pw[q][k] += c[q][j] * t0[k];
+      long double t2[M];
+      for (int k = 0; k < M; ++k) t2[k] = (k ? 2.0L * t1[k - 1] : 0.0L) - t0[k];
+      for (int k = 0; k < M; ++k) {
+        t0[k] = t1[k];
+        t1[k] = t2[k];
+      }
+    }
+    for (int k = 0; k < M; ++k) {
+      tab[p].b[k] = (double)pw[0][BN_DEG - k];
+      tab[p].db[k] = (double)pw[1][BN_DEG - k];
+    }
+  }
+  cudaMemcpyToSymbol(c_bn, tab, sizeof(tab));
+}
+
+// b_n and db/dn for n in [BN_MIN, BN_MAX]
+__device__ __forceinline__ void sersic_bn(double n, double* b_out, double* db_out) {
+  const int p = min(max((int)(4.0f * log2f((float)n * (float)(1.0 / BN_MIN))), 0), BN_PIECES - 1);
+  const BnPiece& t = c_bn[p];
+  const double x = (n - t.mid) * t.inv_half;
+  double b = t.b[0], db = t.db[0];
+#pragma unroll
+  for (int k = 1; k <= BN_DEG; ++k) {
+    b = fma(b, x, t.b[k]);
+    db = fma(db, x, t.db[k]);
+  }
+  *b_out = b;
+  *db_out = db;
 }
 
 // ---------------------------------------------------------------------------
-// prepare: one warp per source, float64, from theta to the SrcPar record
-// (the warp shares the b_n series; lane 0 stores the record)
+// prepare: one thread per source, float64, from theta to the SrcPar record.
+// Bound by the latency of the float64 chain for a few sources and by the thin
+// float64 pipe for many: with a warp of 32 sources every float64 instruction
+// serves all of them (a warp per source issued 32 times as many).  183 -> 9 us
+// for the joint fit's 15 612 sources at a new theta, 23 -> 7 us for a field's
+// 251.  Up to PREPARE_SPREAD sources run as CTAs of one thread instead, so
+// that a warp does not step through the branches of several profile types one
+// after the other (about 2 us per further type).
 // ---------------------------------------------------------------------------
+constexpr int PREPARE_THREADS = 32, PREPARE_SPREAD = 1216;   // 8 CTAs per SM
+
 template <typename T>
-__global__ void prepare_kernel(const SourceDev* __restrict__ srcs, const ImageDev* __restrict__ imgs, int n_src,
-                               const double* __restrict__ theta, SrcPar<T>* __restrict__ par, double* bn_memo,
-                               const int* __restrict__ skip, int* status) {
-  const int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (s >= n_src) return;   // whole warps exit together
+__global__ void __launch_bounds__(PREPARE_THREADS) prepare_kernel(
+    const SourceDev* __restrict__ srcs, const ImageDev* __restrict__ imgs, int n_src, const double* __restrict__ theta,
+    SrcPar<T>* __restrict__ par, const int* __restrict__ skip, int* status) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= n_src) return;
   const SourceDev& sd = srcs[s];
   const ImageDev& im = imgs[sd.image];
   if (skip && skip[im.group]) return;   // the record already holds this point
   double p[MAX_SLOTS];
-  for (int k = 0; k < MAX_SLOTS; ++k) p[k] = (k < sd.nslot) ? (sd.pidx[k] >= 0 ? theta[sd.pidx[k]] : sd.pfix[k]) : 0.0;
+#pragma unroll
+  for (int k = 0; k < MAX_SLOTS; ++k) {
+    const int idx = sd.pidx[k];   // -1 past nslot
+    p[k] = sd.pfix[k];
+    if (idx >= 0) p[k] = theta[idx];
+  }
   SrcPar<T> r;
   memset(&r, 0, sizeof(r));
   r.area = (T)im.area;
@@ -298,32 +344,8 @@ __global__ void prepare_kernel(const SourceDev* __restrict__ srcs, const ImageDe
     double kA = 0.0, amp = 0.0;
     if (ser) {
       double b = 0.0, db = 0.0;
-      int ok = 0;
-      if (n >= 0.05 && n <= 20.0) {
-        // b_n is a function of n alone: a two-entry memo per source (the
-        // current point and the last trial point) keyed on the bits of n.
-        // Every lane reads the same entries, so the branch is warp-uniform.
-        double* mc = bn_memo + 8 * (int64_t)s;
-        const long long key = __double_as_longlong(n);
-        bool hit = false;
-        for (int slot = 0; slot < 2 && !hit; ++slot)
-          if (__double_as_longlong(mc[3 * slot]) == key) {
-            b = mc[3 * slot + 1];
-            db = mc[3 * slot + 2];
-            ok = 1;
-            hit = true;
-          }
-        if (!hit) {
-          sersic_bn(n, &b, &db, &ok);
-          if (ok && (threadIdx.x & 31) == 0) {
-            const int slot = mc[6] == 1.0 ? 1 : 0;   // the older entry (a NaN start reads as 0)
-            mc[3 * slot] = n;
-            mc[3 * slot + 1] = b;
-            mc[3 * slot + 2] = db;
-            mc[6] = 1.0 - slot;
-          }
-        }
-      }
+      const bool ok = n >= BN_MIN && n <= BN_MAX;
+      if (ok) sersic_bn(n, &b, &db);
       good = good && ok;
       amp = im.area * F;
       const double in = 1.0 / n;
@@ -365,17 +387,16 @@ __global__ void prepare_kernel(const SourceDev* __restrict__ srcs, const ImageDe
                    : sd.type == AP_GAUSSIAN ? im.area / (2.0 * M_PI) * (iR * iR) * iq
                                             : im.area * (n - 1.0) / M_PI * (iR * iR) * iq);
   }
-  if ((threadIdx.x & 31) == 0) {
-    if (!good) atomicCAS(status, 0, AP_ERR_NONFINITE);
-    par[s] = r;
-  }
+  if (!good) atomicCAS(status, 0, AP_ERR_NONFINITE);
+  par[s] = r;
 }
 
 template <typename T>
 void launch_prepare(const SourceDev* srcs, const ImageDev* imgs, int n_src, const double* theta, SrcPar<T>* par,
-                    double* bn_memo, const int* skip, int* status, cudaStream_t st) {
+                    const int* skip, int* status, cudaStream_t st) {
   if (n_src <= 0) return;
-  prepare_kernel<T><<<n_src, 32, 0, st>>>(srcs, imgs, n_src, theta, par, bn_memo, skip, status);
+  const int per = n_src <= PREPARE_SPREAD ? 1 : PREPARE_THREADS;
+  prepare_kernel<T><<<(n_src + per - 1) / per, per, 0, st>>>(srcs, imgs, n_src, theta, par, skip, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -1510,9 +1531,9 @@ template void launch_render_samples<float>(const TileWork*, int, const int*, con
                                            const ImageDev*, const int64_t*, const float*, cudaStream_t);
 template void launch_render_samples<double>(const TileWork*, int, const int*, const SourceDev*, const SrcPar<double>*,
                                             const ImageDev*, const int64_t*, const double*, cudaStream_t);
-template void launch_prepare<float>(const SourceDev*, const ImageDev*, int, const double*, SrcPar<float>*, double*,
+template void launch_prepare<float>(const SourceDev*, const ImageDev*, int, const double*, SrcPar<float>*,
                                     const int*, int*, cudaStream_t);
-template void launch_prepare<double>(const SourceDev*, const ImageDev*, int, const double*, SrcPar<double>*, double*,
+template void launch_prepare<double>(const SourceDev*, const ImageDev*, int, const double*, SrcPar<double>*,
                                      const int*, int*, cudaStream_t);
 template void launch_render<float>(int, const TileWork*, int, const int*, const SourceDev*, const SrcPar<float>*, const ImageDev*, const int*, cudaStream_t);
 template void launch_render<double>(int, const TileWork*, int, const int*, const SourceDev*, const SrcPar<double>*, const ImageDev*, const int*, cudaStream_t);

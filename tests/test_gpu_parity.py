@@ -764,3 +764,18 @@ def test_live_psf_lm_iterations_follow_the_oracle():
     c_ref = O.chi2(pr, th_ref)[0]
     assert abs(_np(chi2)[0] - c_ref) <= 1e-8 * c_ref
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("n", [0.05, 0.0594603557, 0.0594603558, 0.36, 0.5, 1.0, 2.9999, 8.0, 19.027313, 19.027314, 20.0])
+def test_sersic_bn_table(n):
+    """b_n and db/dn from the piecewise table at its ends and around piece
+    edges (quarter octaves from 0.05): chi^2 and the gradient of the float64
+    form against the oracle's own root (the tolerances of the other float64
+    comparisons)."""
+    pr = problem("single_sersic", H=40, W=37)
+    theta = np.array([18.3, 20.8, 0.7, 0.6, n, 6.0, 10.0, 1.0])
+    ctx = device_context(pr, "f64")
+    c, g = ctx.eval(theta)
+    np.testing.assert_allclose(_np(c), O.chi2(pr, theta), rtol=TOL_F64, atol=0)
+    assert_grad_close(_np(g), O.gradient(pr, theta), grad_scale(pr, theta), 1e-8)
+    assert ctx.status() == 0
