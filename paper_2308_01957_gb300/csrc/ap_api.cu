@@ -100,9 +100,6 @@ struct ap_ctx {
   int* d_jt_src = nullptr;
   GramPlan gplan{};
   std::vector<GramRange> gram_ranges;
-  std::vector<int> h_tile_ncol;   // columns of every Gram tile (sorted)
-  int gram_tc_min = 0;            // float path: tiles with tc_min .. tc_max columns run on tcgen05
-  int gram_tc_max = 0;
   void* d_dbuf = nullptr;
   int64_t dbuf_elems = 0;
   std::vector<int64_t> h_row_ptr;
@@ -272,8 +269,6 @@ void free_problem(ap_ctx* c) {
   c->d_live_imgs = nullptr;
   c->n_live = 0;
   c->n_src_user = 0;
-  c->h_tile_ncol.clear();
-  c->gram_tc_min = GRAM_TC_MIN_DEFAULT;
 }
 
 // Parameter box applied after each LM update: q in [0.05, 1], Sersic n in
@@ -327,7 +322,8 @@ int do_eval(ap_ctx* c, const double* theta, double* chi2_out, double* grad_out, 
   {
     Bracket b(c, st, "forward_conv_chi2");
     launch_forward_conv<T>(c->conv_variant, c->d_fwork, c->frange.data(), (int)c->frange.size(), c->d_imgs,
-                           c->d_chi2_partial, model_ptrs_dev, skip, trial ? 1 : 0, c->d_status, c->Kmax, st);
+                           c->d_chi2_partial, model_ptrs_dev, skip, trial ? 1 : 0, want_D ? 1 : 0, c->d_status,
+                           c->Kmax, st);
   }
   if (chi2_out) {
     Bracket b(c, st, "chi2_gather");
@@ -348,7 +344,7 @@ int do_eval(ap_ctx* c, const double* theta, double* chi2_out, double* grad_out, 
       Bracket b(c, st, "render_adjoint");
       launch_render_adjoint<T>(c->opt.quad_order, c->d_rwork, c->n_rwork, c->d_tile_src, c->d_srcs,
                                (const SrcPar<T>*)c->d_par, c->d_imgs, c->d_grad_partial,
-                               want_D ? (T*)c->d_dbuf : nullptr, st);
+                               want_D ? (T*)c->d_dbuf : nullptr, want_D && !c->f64 ? (T*)c->d_jbuf : nullptr, st);
     }
     {
       Bracket b(c, st, "grad_gather");
@@ -577,7 +573,7 @@ void eval_shifted(ap_ctx* c, const double* theta, int method, double* chi2_out, 
   {
     Bracket b(c, st, "forward_conv_chi2");
     launch_forward_conv<T>(c->conv_variant, c->d_fwork, c->frange.data(), (int)c->frange.size(), c->d_imgs,
-                           c->d_chi2_partial, model_out ? c->d_model_ptrs : nullptr, nullptr, 0, c->d_status,
+                           c->d_chi2_partial, model_out ? c->d_model_ptrs : nullptr, nullptr, 0, 0, c->d_status,
                            c->Kmax, st);
   }
   if (chi2_out) {
@@ -610,7 +606,7 @@ void eval_adaptive(ap_ctx* c, const double* theta, double tol, double* chi2_out,
   {
     Bracket b(c, st, "forward_conv_chi2");
     launch_forward_conv<T>(c->conv_variant, c->d_fwork, c->frange.data(), (int)c->frange.size(), c->d_imgs,
-                           c->d_chi2_partial, model_out ? c->d_model_ptrs : nullptr, nullptr, 0, c->d_status,
+                           c->d_chi2_partial, model_out ? c->d_model_ptrs : nullptr, nullptr, 0, 0, c->d_status,
                            c->Kmax, st);
   }
   if (chi2_out) {
@@ -748,28 +744,6 @@ void ap_destroy(ap_ctx* c) {
 }
 
 const char* ap_get_error(ap_ctx* c) { return c ? c->err.c_str() : ""; }
-
-// The Gram's column blocking per run of tiles (sorted by column count): the
-// float path sends tiles of tc_min .. min(tc_max, gram_tc_max_cols()) columns
-// to the tcgen05 kernel (in the form for up to 32, 64 or 128 columns) and the
-// others to the warp-MMA kernel (column blocks of up to 96); the float64 path
-// blocks by 32.
-std::vector<GramRange> gram_ranges_for(const std::vector<int>& tile_ncol, bool f64, int tc_min,
-                                       int tc_max = 1 << 30) {
-  std::vector<GramRange> out;
-  for (size_t t = 0; t < tile_ncol.size(); ++t) {
-    GramRange gr{(int)t, (int)t + 1, 0, 0, 0};
-    if (f64) gram_blocking<double>(tile_ncol[t], &gr.cb, &gr.two);
-    else if (tile_ncol[t] >= tc_min && tile_ncol[t] <= std::min(tc_max, gram_tc_max_cols()))
-      gr.tc = gram_tc_kind(tile_ncol[t]);
-    else gram_blocking<float>(tile_ncol[t], &gr.cb, &gr.two);
-    if (!out.empty() && out.back().cb == gr.cb && out.back().two == gr.two && out.back().tc == gr.tc)
-      out.back().t1++;
-    else
-      out.push_back(gr);
-  }
-  return out;
-}
 
 int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_source_desc* srcs, int n_src,
                    int n_params, void* stream) {
@@ -1018,11 +992,17 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
     bool any_free = false;
     for (int k = 0; k < m.nslot; ++k) any_free |= m.pidx[k] >= 0;
     const int64_t area = (int64_t)(m.box[1] - m.box[0]) * (m.box[3] - m.box[2]);
-    m.j_off = -1;
+    m.j_off = m.g_off = -1;
+    m.nfree = 0;
+    for (int k = 0; k < m.nslot; ++k) m.nfree += m.pidx[k] >= 0;
     m.sup[0] = m.sup[1] = m.sup[2] = m.sup[3] = 0;
     if (any_free && area > 0) {
-      m.d_off = dbuf_elems;
-      dbuf_elems += area * m.nslot;
+      // float path: an unconvolved source's derivatives go straight to its
+      // column blocks
+      if (f64 || m.conv) {
+        m.d_off = dbuf_elems;
+        dbuf_elems += area * m.nslot;
+      }
       const ImageDev& im = I[m.image];
       const int hh = m.conv ? im.h : 0;
       m.sup[0] = std::max(m.box[0] - hh, 0);
@@ -1031,26 +1011,31 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
       m.sup[3] = std::min(m.box[3] + hh, im.W);
       if (m.sup[0] >= m.sup[1] || m.sup[2] >= m.sup[3]) m.sup[0] = m.sup[1] = m.sup[2] = m.sup[3] = 0;
       const int64_t sarea = (int64_t)(m.sup[1] - m.sup[0]) * (m.sup[3] - m.sup[2]);
-      if (m.conv && sarea > 0) {
+      if (f64 && m.conv && sarea > 0) {
         m.j_off = jbuf_elems;
         jbuf_elems += sarea * m.nslot;
+      }
+      if (!f64 && sarea > 0) {
+        m.gt[0] = m.sup[0] / TILE;
+        m.gt[1] = m.sup[2] / TILE;
+        m.gt[2] = (m.sup[3] - 1) / TILE - m.gt[1] + 1;
+        m.g_off = jbuf_elems;
+        jbuf_elems += (int64_t)((m.sup[1] - 1) / TILE - m.gt[0] + 1) * m.gt[2] * m.nfree * TILE_THREADS;
       }
     }
   }
   std::vector<TileWork> jwork;
   std::vector<int> jt_src, tile_ncol;
-  int gram_cols = 4;
   std::vector<std::vector<int>> rows_of(n_params);
   {
     std::set<std::pair<int, int>> src_pairs;
-    gram_cols = 4;
     for (int i = 0; i < n_img; ++i) {
       const ImageDev& m = I[i];
       const int nr = (m.H + TILE - 1) / TILE, nc = (m.W + TILE - 1) / TILE;
       std::vector<std::vector<int>> lists((size_t)nr * nc);
       for (int s = 0; s < n_src; ++s) {
         const SourceDev& sd = S[s];
-        if (sd.image != i || sd.d_off < 0) continue;
+        if (sd.image != i || (f64 ? sd.d_off : sd.g_off) < 0) continue;
         const int r0 = sd.sup[0], r1 = sd.sup[1], c0 = sd.sup[2], c1 = sd.sup[3];
         if (r0 >= r1 || c0 >= c1) continue;
         for (int tr = r0 / TILE; tr <= (r1 - 1) / TILE; ++tr)
@@ -1060,11 +1045,6 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
         for (int tc = 0; tc < nc; ++tc) {
           auto& L = lists[(size_t)tr * nc + tc];
           if (L.empty()) continue;
-          int ncol = 0;
-          for (int s : L)
-            for (int k = 0; k < S[s].nslot; ++k) ncol += S[s].pidx[k] >= 0;
-
-          gram_cols = std::max(gram_cols, ncol);
           TileWork w{i, 1, tr * TILE, tc * TILE, (int)jt_src.size(), 0};
           jt_src.insert(jt_src.end(), L.begin(), L.end());
           w.e1 = (int)jt_src.size();
@@ -1086,11 +1066,9 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
       }
     }
     // tiles by free-column class (largest first), in image order within a
-    // class: the Gram launches one column blocking per run of tiles, and
-    // tiles that run side by side are neighbours sharing column images (in
-    // the L2, and in the address translation caches).  A class is 16 columns
-    // wide in the float path (its column blocks and tensor-core thresholds
-    // are multiples of 16), 4 in the float64 path (blocks of 4 up to 32)
+    // class: the Gram launches one column blocking per class.  A class is 16
+    // columns wide in the float path (its kernel forms are multiples of 16), 4
+    // in the float64 path (blocks of 4 up to 32)
     std::vector<int> ncol_of(jwork.size());
     for (size_t t = 0; t < jwork.size(); ++t) {
       int nc = 0;
@@ -1126,9 +1104,9 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
   }
 
   // ---- J^T W J plan: source pairs per tile, scratch blocks, CSR positions ----
-  std::vector<int64_t> g_tab0(jwork.size() + 1, 0), g_tab, g_col_ptr;
-  std::vector<GramCol> g_cols;
-  std::vector<int> g_tabs;
+  std::vector<int64_t> g_tab0(jwork.size() + 1, 0), g_tab;
+  std::vector<GramEnt> g_ents;
+  std::vector<GramJob> g_jobs;
   std::vector<GramPair> g_pairs;
   std::vector<GramRange> g_ranges;
   int g_n_light = 0;
@@ -1170,42 +1148,27 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
         }
     }
     g_tab0[jwork.size()] = (int64_t)g_tab.size();
-    // float path: every tile's free columns in (source, slot) order, as the
-    // tensor-core tile Gram reads them (it then skips building the list)
+    // float path: where each source of a tile's list keeps the tile's columns
     if (!f64) {
-      g_col_ptr.assign(jwork.size() + 1, 0);
-      for (size_t t = 0; t < jwork.size(); ++t) {
-        const TileWork& w = jwork[t];
+      g_ents.reserve(jt_src.size());
+      for (const TileWork& w : jwork) {
+        int col0 = 0;
         for (int e = w.e0; e < w.e1; ++e) {
           const SourceDev& sd = S[jt_src[e]];
-          int nf = 0;
-          for (int k = 0; k < sd.nslot; ++k) nf += sd.pidx[k] >= 0;
-          const int* bx = sd.conv ? sd.sup : sd.box;
-          const int bw = bx[3] - bx[2];
-          const int64_t area = (int64_t)(bx[1] - bx[0]) * bw;
-          auto clampt = [](int v) { return (uint32_t)(v < 0 ? 0 : (v > TILE ? TILE : v)); };
-          const uint32_t bounds = clampt(bx[0] - w.r0) | (clampt(bx[1] - w.r0) << 8) | (clampt(bx[2] - w.c0) << 16) |
-                                  (clampt(bx[3] - w.c0) << 24);
-          const int off0 = (w.r0 - bx[0]) * bw + (w.c0 - bx[2]);
-          const int64_t base = sd.conv ? sd.j_off : sd.d_off;
-          int f = 0;
-          for (int k = 0; k < sd.nslot; ++k) {
-            if (sd.pidx[k] < 0) continue;
-            g_cols.push_back(GramCol{base + k * area, off0, bw, bounds,
-                                     ((e - w.e0) << 8) | (f << 4) | nf | (sd.conv ? GRAM_COL_CONV : 0)});
-            ++f;
-          }
+          g_ents.resize(std::max<size_t>(g_ents.size(), (size_t)e + 1));
+          g_ents[e] = GramEnt{col_block(sd, 0, w.r0, w.c0), sd.nfree, col0};
+          col0 += sd.nfree;
         }
-        g_col_ptr[t + 1] = (int64_t)g_cols.size();
       }
     }
-    // light pairs first (tile-major blocks), heavy pairs after (entry-major)
+    auto light_pair = [](const GramPair& gp) { return (int64_t)gp.cnt * gp.ma * gp.mb <= GRAM_LIGHT_VALUES; };
+    // light pairs first (a warp sums each), the others after (cut into runs)
     std::vector<int> new_id(g_pairs.size());
     {
       std::vector<GramPair> light, heavy;
       std::vector<int> lA, lB, hA, hB;
       for (size_t q = 0; q < g_pairs.size(); ++q) {
-        const bool hv = g_pairs[q].cnt > GRAM_HEAVY_TILES;
+        const bool hv = !light_pair(g_pairs[q]);
         new_id[q] = (int)(hv ? heavy.size() : light.size());
         (hv ? heavy : light).push_back(g_pairs[q]);
         (hv ? hA : lA).push_back(pA[q]);
@@ -1213,7 +1176,7 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
       }
       g_n_light = (int)light.size();
       for (size_t q = 0; q < g_pairs.size(); ++q)
-        if (g_pairs[q].cnt > GRAM_HEAVY_TILES) new_id[q] += g_n_light;
+        if (!light_pair(g_pairs[q])) new_id[q] += g_n_light;
       light.insert(light.end(), heavy.begin(), heavy.end());
       lA.insert(lA.end(), hA.begin(), hA.end());
       lB.insert(lB.end(), hB.begin(), hB.end());
@@ -1225,20 +1188,25 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
       gp.base = g_scr;
       g_scr += (int64_t)gp.cnt * gp.ma * gp.mb;
     }
-    g_tabs.resize(g_tab.size());
     for (size_t k = 0; k < g_tab.size(); ++k) {
-      const int id = new_id[g_tab[k]];
-      const GramPair& gp = g_pairs[id];
-      const bool hv = id >= g_n_light;
-      g_tab[k] = gp.base + (int64_t)rank_of[k] * (hv ? 1 : gp.ma * gp.mb);
-      g_tabs[k] = hv ? gp.cnt : 1;
+      const GramPair& gp = g_pairs[new_id[g_tab[k]]];
+      g_tab[k] = gp.base + (int64_t)rank_of[k] * (gp.ma * gp.mb);
     }
     std::vector<int>().swap(rank_of);
-    // column blocking per run of tiles (the tiles are sorted by column count);
-    // the float path's threshold between the warp-MMA and the tcgen05 kernel
-    // is chosen by timing once the plans are on the device
-    g_ranges = gram_ranges_for(tile_ncol, f64, GRAM_TC_MIN_DEFAULT);
-    c->h_tile_ncol = tile_ncol;
+    // the launches: jobs by kernel form (float path), runs of tiles sharing
+    // one column blocking (float64 path)
+    if (!f64) {
+      gram_plan_jobs(jwork, g_tab0, tile_ncol, g_jobs, g_ranges);
+    } else {
+      for (size_t t = 0; t < tile_ncol.size(); ++t) {
+        GramRange gr{(int)t, (int)t + 1, 0, 0};
+        gram64_blocking(tile_ncol[t], &gr.form, &gr.two);
+        if (!g_ranges.empty() && g_ranges.back().form == gr.form && g_ranges.back().two == gr.two)
+          g_ranges.back().t1++;
+        else
+          g_ranges.push_back(gr);
+      }
+    }
     // CSR positions of every block entry and its mirror; entries below the
     // diagonal of a source's own block are left out (their mirror is there)
     auto find = [&](int r, int cc) -> int64_t {
@@ -1570,6 +1538,10 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
     if ((rc = dev_alloc(c, &m.unc, (size_t)m.H * m.W * tsz))) return rc;
     if ((rc = dev_alloc(c, &m.wr, (size_t)m.H * m.W * tsz))) return rc;
     if ((rc = dev_alloc(c, &m.wr_trial, (size_t)m.H * m.W * tsz))) return rc;
+    if (!f64) {
+      if ((rc = dev_alloc(c, (void**)&m.sw, (size_t)m.H * m.W * sizeof(float)))) return rc;
+      CUDA_TRY(c, cudaMemset(m.sw, 0, (size_t)m.H * m.W * sizeof(float)));
+    }
   }
   if ((rc = upload(c, &c->d_live_imgs, live_imgs))) return rc;
   c->n_live = (int)live_imgs.size();
@@ -1621,41 +1593,43 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
   if ((rc = upload(c, &c->d_jt_src, jt_src))) return rc;
   {
     const int64_t *d_t0, *d_tab, *d_pos;
-    const int* d_tabs;
     const GramPair* d_gp;
+    const GramJob* d_jobs;
+    const GramEnt* d_ents;
+    const GramRun* d_runs;
     if ((rc = upload(c, &d_t0, g_tab0))) return rc;
     if ((rc = upload(c, &d_tab, g_tab))) return rc;
-    if ((rc = upload(c, &d_tabs, g_tabs))) return rc;
     if ((rc = upload(c, &d_pos, g_pos))) return rc;
     if ((rc = upload(c, &d_gp, g_pairs))) return rc;
-    double* d_scr;
-    if ((rc = dev_alloc(c, (void**)&d_scr, (size_t)std::max<int64_t>(g_scr, 1) * sizeof(double)))) return rc;
-    // work list of the heavy-pair reduction: one item per stored entry, the
-    // entries spanning more than GRAM_CTA_TILES tiles first (a CTA each)
-    std::vector<int> items, warp_items;
+    if ((rc = upload(c, &d_jobs, g_jobs))) return rc;
+    if ((rc = upload(c, &d_ents, g_ents))) return rc;
+    void* d_scr;
+    static_assert(sizeof(float2) == sizeof(double), "scratch values of either path");
+    if ((rc = dev_alloc(c, &d_scr, (size_t)std::max<int64_t>(g_scr, 1) * sizeof(double)))) return rc;
+    // entries below the diagonal of a source's own block are never stored
+    // (the sums of pass 2 that read them are dropped): defined values
+    CUDA_TRY(c, cudaMemset(d_scr, 0, (size_t)std::max<int64_t>(g_scr, 1) * sizeof(double)));
+    std::vector<GramRun> runs;
     for (int q = g_n_light; q < (int)g_pairs.size(); ++q) {
       const GramPair& gp = g_pairs[q];
-      for (int e = 0; e < gp.ma * gp.mb; ++e)
-        if (g_pos[gp.pos + 2 * e] >= 0)
-          (gp.cnt > GRAM_CTA_TILES ? items : warp_items).push_back(((q - g_n_light) << 6) | e);
+      const int per = std::max(1, GRAM_RUN_VALUES / (gp.ma * gp.mb)), n = (gp.cnt + per - 1) / per;
+      const int first = (int)runs.size();
+      for (int k = 0; k < n; ++k) runs.push_back(GramRun{q, k * per, std::min(gp.cnt, (k + 1) * per), first, k, n});
     }
-    const int n_heavy_cta = (int)items.size();
-    items.insert(items.end(), warp_items.begin(), warp_items.end());
-    const int* d_items;
-    if ((rc = upload(c, &d_items, items))) return rc;
-    const int64_t* d_col_ptr = nullptr;
-    const GramCol* d_cols = nullptr;
-    if (!f64) {
-      if ((rc = upload(c, &d_col_ptr, g_col_ptr))) return rc;
-      if ((rc = upload(c, &d_cols, g_cols))) return rc;
-    }
-    std::vector<GramCol>().swap(g_cols);
-    c->gplan = GramPlan{d_t0, d_tab, d_tabs, d_scr, d_gp, d_pos, g_n_light, (int)g_pairs.size() - g_n_light,
-                        d_items, (int)items.size(), n_heavy_cta, d_col_ptr, d_cols};
+    double* d_part;
+    int* d_done;
+    if ((rc = upload(c, &d_runs, runs))) return rc;
+    if ((rc = dev_alloc(c, (void**)&d_part, std::max<size_t>(runs.size(), 1) * 64 * sizeof(double)))) return rc;
+    if ((rc = dev_alloc(c, (void**)&d_done, std::max<size_t>(runs.size(), 1) * sizeof(int)))) return rc;
+    CUDA_TRY(c, cudaMemset(d_done, 0, std::max<size_t>(runs.size(), 1) * sizeof(int)));
+    c->gplan = GramPlan{d_t0, d_tab, d_scr, d_gp, d_pos, g_n_light, d_runs, (int)runs.size(), d_part, d_done,
+                        d_jobs, d_ents};
     c->gram_ranges = g_ranges;
   }
   if ((rc = dev_alloc(c, &c->d_dbuf, (size_t)std::max<int64_t>(dbuf_elems, 1) * tsz))) return rc;
   if ((rc = dev_alloc(c, &c->d_jbuf, (size_t)std::max<int64_t>(jbuf_elems, 1) * tsz))) return rc;
+  // column blocks: the pixels outside the supports stay zero
+  if (!f64) CUDA_TRY(c, cudaMemset(c->d_jbuf, 0, (size_t)std::max<int64_t>(jbuf_elems, 1) * tsz));
   if ((rc = upload(c, &c->d_row_ptr, row_ptr))) return rc;
   if ((rc = upload(c, &c->d_col_idx, col_idx))) return rc;
   if ((rc = dev_alloc(c, (void**)&c->d_vals, std::max<size_t>(col_idx.size(), 1) * sizeof(double)))) return rc;
@@ -1741,14 +1715,10 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
   int vok[N_CONV_VARIANTS] = {};
   if (f64) {
     configure_conv<double>(Kmax, vok);
-    configure_gram<double>(0);
-
   } else {
     configure_conv<float>(Kmax, vok);
-    configure_gram<float>(0);
-    configure_gram_tc();
-
   }
+  if (!configure_gram(f64)) return fail(c, AP_ERR_CUDA, "Gram kernels cannot get their shared memory");
   configure_solve();
   if (!live_imgs.empty() && !configure_live(Kmax, f64 ? 1 : 0))
     return fail(c, AP_ERR_ARG, "the live PSF's column kernel does not fit the PSF size in shared memory");
@@ -1792,11 +1762,11 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
         const auto& ar = c->v_arange[v];
         if (f64) {
           launch_forward_conv<double>(v, c->v_fwork[v], fr.data(), (int)fr.size(), c->d_imgs, c->d_chi2_partial, nullptr,
-                                      nullptr, 0, c->d_status, Kmax, st);
+                                      nullptr, 0, 0, c->d_status, Kmax, st);
           launch_adjoint_conv<double>(v, c->v_awork[v], ar.data(), (int)ar.size(), c->d_imgs, Kmax, st);
         } else {
           launch_forward_conv<float>(v, c->v_fwork[v], fr.data(), (int)fr.size(), c->d_imgs, c->d_chi2_partial, nullptr,
-                                     nullptr, 0, c->d_status, Kmax, st);
+                                     nullptr, 0, 0, c->d_status, Kmax, st);
           launch_adjoint_conv<float>(v, c->v_awork[v], ar.data(), (int)ar.size(), c->d_imgs, Kmax, st);
         }
         cudaEventRecord(e1, st);
@@ -1828,7 +1798,7 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
     std::vector<JcolWork> jc;
     for (int s = 0; s < n_src; ++s) {
       const SourceDev& m = S[s];
-      if (m.j_off < 0) continue;
+      if (!m.conv || (f64 ? m.j_off : m.g_off) < 0) continue;
       for (int r = m.sup[0]; r < m.sup[1]; r += TH)
         for (int cc = m.sup[2]; cc < m.sup[3]; cc += TW) jc.push_back(JcolWork{s, r, cc});
     }
@@ -1852,7 +1822,7 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
     bool all = true;
     for (int s = 0; s < n_src; ++s) {
       const SourceDev& m = S[s];
-      if (m.j_off < 0) continue;
+      if (!m.conv || (f64 ? m.j_off : m.g_off) < 0) continue;
       const ImageDev& im = I[m.image];
       if (!im.spec64 && !im.spec128) { all = false; continue; }
       // block size with the smaller estimated cost: blocks x N^2 log2 N
@@ -1872,7 +1842,7 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
       for (int a = 0; a < nf; ++a)
         for (int r = m.sup[0]; r < m.sup[1]; r += B)
           for (int cc = m.sup[2]; cc < m.sup[3]; cc += B)
-            jf[N == 128].push_back(JcolFftWork{s, fs[a], r - m.box[0], cc - m.box[2]});
+            jf[N == 128].push_back(JcolFftWork{s, fs[a], a, r - m.box[0], cc - m.box[2]});
     }
     if (all) {
       c->n_jf64 = (int)jf[0].size();
@@ -1906,51 +1876,6 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
       c->jcol_fft = c->opt.jcol_mode == AP_JCOL_FFT || (c->opt.jcol_mode == AP_JCOL_AUTO && t[1] < t[0]);
     }
   }
-  // the Gram's tcgen05 threshold: tiles with few columns cost the tensor-core
-  // kernel its per-tile hand-overs for little work, so both kernels are timed
-  // on this problem's tiles for a few thresholds and the fastest kept
-  // a forced threshold starts a 16-column class (tiles are grouped by class)
-  c->gram_tc_min = c->opt.gram_tc_min > 0 ? (c->opt.gram_tc_min + 14) / 16 * 16 + 1 : GRAM_TC_MIN_DEFAULT;
-  c->gram_tc_max = gram_tc_max_cols();
-  if (c->opt.gram_tc_min > 0 && !f64) c->gram_ranges = gram_ranges_for(c->h_tile_ncol, false, c->gram_tc_min);
-  if (!f64 && !c->h_tile_ncol.empty() && c->opt.gram_tc_min <= 0) {
-    // (tc_min, tc_max): the tensor-core kernel for tiles of tc_min .. tc_max
-    // columns; the 128-column form runs fewer CTAs per SM, so the warp-MMA
-    // kernel may serve tiles past 64 columns better
-    const int none = gram_tc_max_cols() + 1;
-    const int cands[][2] = {{1, 128}, {33, 128}, {49, 128}, {65, 128}, {97, 128}, {1, 64}, {33, 64}, {49, 64},
-                            {none, 128}};
-    cudaEvent_t e0, e1;
-    CUDA_TRY(c, cudaEventCreate(&e0));
-    CUDA_TRY(c, cudaEventCreate(&e1));
-    double best = 1e300;
-    for (const auto& cd : cands) {
-      const std::vector<GramRange> rg = gram_ranges_for(c->h_tile_ncol, false, cd[0], cd[1]);
-      double tot = 0.0;
-      for (int rep = 0; rep < 3; ++rep) {
-        cudaEventRecord(e0, st);
-        launch_gram<float>(c->d_jwork, rg.data(), (int)rg.size(), c->d_jt_src, c->d_srcs, c->d_imgs,
-                           (const float*)c->d_dbuf, (const float*)c->d_jbuf, c->gplan, c->d_vals, c->d_status, st,
-                           c->have_fj ? &c->fj : nullptr);
-        cudaEventRecord(e1, st);
-        CUDA_TRY(c, cudaEventSynchronize(e1));
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (rep > 0) tot += ms;
-      }
-      if (tot < best) {
-        best = tot;
-        c->gram_tc_min = cd[0];
-        c->gram_tc_max = cd[1];
-      }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    CUDA_TRY(c, cudaGetLastError());
-    CUDA_TRY(c, cudaMemset(c->d_status, 0, sizeof(int)));
-    c->gram_ranges = gram_ranges_for(c->h_tile_ncol, false, c->gram_tc_min, c->gram_tc_max);
-  }
-
   c->h_imgs = I;
   c->h_srcs = S;
   c->n_img = n_img;

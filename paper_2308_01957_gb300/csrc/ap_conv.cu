@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(BX * BY) forward_conv_kernel(const ConvWork* _
                                                                double* __restrict__ chi2_partial,
                                                                void* const* __restrict__ model_out,
                                                                const int* __restrict__ skip, int trial,
-                                                               int* __restrict__ status) {
+                                                               int store_sw, int* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* smem = reinterpret_cast<T*>(smem_raw);
   __shared__ double red[32];
@@ -225,6 +225,8 @@ __global__ void __launch_bounds__(BX * BY) forward_conv_kernel(const ConvWork* _
         const T wr = wt * r;
         c2t += wr * r;
         WR[o] = wr;
+        // sqrt(w) for the Jacobian columns (correctly rounded division and root)
+        if (sizeof(T) == 4 && store_sw) im.sw[o] = wt > (T)0 ? 1.0f / sqrtf((float)var) : 0.f;
       }
     }
   }
@@ -272,7 +274,8 @@ __global__ void __launch_bounds__(BX * BY) adjoint_conv_kernel(const ConvWork* _
 // Jacobian columns of convolved sources: J_k = P * (d G_s / d theta_k) on the
 // source's Jacobian support (its sampling box grown by h, clipped to the
 // image), from the stored derivative images.  One CTA per output tile of one
-// source, looping over the source's free slots.
+// source, looping over the source's free slots.  The float path stores
+// sqrt(w) J_k into the column blocks, the float64 path J_k row by row.
 template <typename T, int BX, int BY, int RY, int NC>
 __global__ void __launch_bounds__(BX * BY) jcol_kernel(const JcolWork* __restrict__ work,
                                                        const SourceDev* __restrict__ srcs,
@@ -288,12 +291,12 @@ __global__ void __launch_bounds__(BX * BY) jcol_kernel(const JcolWork* __restric
   const int sh = sd.sup[1] - sd.sup[0], sw = sd.sup[3] - sd.sup[2];
   const int64_t sarea = (int64_t)sh * sw;
   const int lx = threadIdx.x % BX, ly = threadIdx.x / BX;
+  int f = 0;
   for (int k = 0; k < sd.nslot; ++k) {
     if (sd.pidx[k] < 0) continue;
     T acc[RY][RX];
     corr_any<T, BX, BY, RY, NC>(dbuf + sd.d_off + k * barea, bh, bw, w.r0 - im.h - sd.box[0],
                                 w.c0 - im.h - sd.box[2], (const T*)im.psf_flip, im.K, im.K4, smem, acc);
-    T* out = jbuf + sd.j_off + k * sarea;
 #pragma unroll
     for (int ry = 0; ry < RY; ++ry) {
       const int oi = w.r0 + ly * RY + ry;
@@ -301,9 +304,14 @@ __global__ void __launch_bounds__(BX * BY) jcol_kernel(const JcolWork* __restric
 #pragma unroll
       for (int rx = 0; rx < RX; ++rx) {
         const int oj = w.c0 + lx * RX + rx;
-        if (oj < sd.sup[3]) out[(int64_t)(oi - sd.sup[0]) * sw + (oj - sd.sup[2])] = acc[ry][rx];
+        if (oj >= sd.sup[3]) break;
+        if constexpr (sizeof(T) == 4)
+          jbuf[col_block(sd, f, oi, oj)] = acc[ry][rx] * im.sw[(size_t)oi * im.W + oj];
+        else
+          jbuf[sd.j_off + k * sarea + (int64_t)(oi - sd.sup[0]) * sw + (oj - sd.sup[2])] = acc[ry][rx];
       }
     }
+    ++f;
     __syncthreads();   // the next slot reloads the shared tile
   }
 }
@@ -412,10 +420,10 @@ int conv_variant_fast(int v) {
 
 template <typename T, int BX, int BY, int RY, int NC>
 static void fwd_launch(const ConvWork* work, int n, const ImageDev* imgs, double* chi2_partial, void* const* model_out,
-                       const int* skip, int trial, int* status, int kmax, cudaStream_t st) {
+                       const int* skip, int trial, int store_sw, int* status, int kmax, cudaStream_t st) {
   if constexpr (NC == 0 || (sizeof(T) == 4 && fast_shape(BX, BY, RY)))
     forward_conv_kernel<T, BX, BY, RY, NC><<<n, BX * BY, corr_smem_bytes<T, BX, BY, RY>(kmax), st>>>(
-        work, imgs, chi2_partial, model_out, skip, trial, status);
+        work, imgs, chi2_partial, model_out, skip, trial, store_sw, status);
 }
 template <typename T, int BX, int BY, int RY, int NC>
 static void adj_launch(const ConvWork* work, int n, const ImageDev* imgs, int kmax, cudaStream_t st) {
@@ -434,13 +442,13 @@ static void jc_launch(const JcolWork* work, int n, const SourceDev* srcs, const 
 // (ranges[k] = {nc, start, count}); nc = 0 runs the generic tile.
 template <typename T>
 void launch_forward_conv(int v, const ConvWork* work, const ConvRange* ranges, int n_ranges, const ImageDev* imgs,
-                         double* chi2_partial, void* const* model_out, const int* skip, int trial, int* status,
-                         int kmax, cudaStream_t st) {
+                         double* chi2_partial, void* const* model_out, const int* skip, int trial, int store_sw,
+                         int* status, int kmax, cudaStream_t st) {
   for (int k = 0; k < n_ranges; ++k) {
     const ConvRange r = ranges[k];
     if (r.count <= 0) continue;
     const int nc = conv_variant_fast(v) ? r.nc : 0;
-#define AP_FWD_NC(NC, BX, BY, RY) fwd_launch<T, BX, BY, RY, NC>(work + r.start, r.count, imgs, chi2_partial + r.start, model_out, skip, trial, status, kmax, st)
+#define AP_FWD_NC(NC, BX, BY, RY) fwd_launch<T, BX, BY, RY, NC>(work + r.start, r.count, imgs, chi2_partial + r.start, model_out, skip, trial, store_sw, status, kmax, st)
 #define AP_FWD(BX, BY, RY, dummy) AP_NC_SWITCH(T, nc, AP_FWD_NC, BX, BY, RY)
     AP_CONV_SWITCH(v, AP_FWD, 0)
 #undef AP_FWD
@@ -533,8 +541,8 @@ template void configure_conv<float>(int, int*);
 template void configure_conv<double>(int, int*);
 template void launch_jcol<float>(int, const JcolWork*, const ConvRange*, int, const SourceDev*, const ImageDev*, const float*, float*, int, cudaStream_t);
 template void launch_jcol<double>(int, const JcolWork*, const ConvRange*, int, const SourceDev*, const ImageDev*, const double*, double*, int, cudaStream_t);
-template void launch_forward_conv<float>(int, const ConvWork*, const ConvRange*, int, const ImageDev*, double*, void* const*, const int*, int, int*, int, cudaStream_t);
-template void launch_forward_conv<double>(int, const ConvWork*, const ConvRange*, int, const ImageDev*, double*, void* const*, const int*, int, int*, int, cudaStream_t);
+template void launch_forward_conv<float>(int, const ConvWork*, const ConvRange*, int, const ImageDev*, double*, void* const*, const int*, int, int, int*, int, cudaStream_t);
+template void launch_forward_conv<double>(int, const ConvWork*, const ConvRange*, int, const ImageDev*, double*, void* const*, const int*, int, int, int*, int, cudaStream_t);
 template void launch_adjoint_conv<float>(int, const ConvWork*, const ConvRange*, int, const ImageDev*, int, cudaStream_t);
 template void launch_adjoint_conv<double>(int, const ConvWork*, const ConvRange*, int, const ImageDev*, int, cudaStream_t);
 

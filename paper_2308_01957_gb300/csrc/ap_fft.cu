@@ -316,19 +316,24 @@ __global__ void __launch_bounds__(FftShape<N>::NTR, FftShape<N>::MINB) jcol_fft_
   fft_lines<N, NT, 1, LDA, true>(sm, H, tw, ld_pack, st_a);
   __syncthreads();
   // outputs: block rows / columns [0, B) sit at [K - 1, N) of the circular
-  // result; thread t takes column t mod N of rows t / N, t / N + NT / N, ...
-  const int sw = sd.sup[3] - sd.sup[2];
-  float* o1 = jbuf + sd.j_off + w.k * (int64_t)(sd.sup[1] - sd.sup[0]) * sw;
+  // result; thread t takes column t mod N of rows t / N, t / N + NT / N, ...,
+  // stored sqrt(w)-scaled into the source's column blocks
   constexpr int RSTEP = NT / N;   // rows per sweep (the threads past RSTEP * N idle)
   const int j = threadIdx.x % N;
   const int oj = sd.box[2] + w.bx0 + j;
   if (threadIdx.x < RSTEP * N && j < B && oj >= sd.sup[2] && oj < sd.sup[3]) {
-    for (int i = threadIdx.x / N; i < B; i += RSTEP) {
-      const int oi = sd.box[0] + w.by0 + i;
-      if (oi < sd.sup[0] || oi >= sd.sup[1]) continue;
-      const int rho = i + K - 1;
-      const float2 z = sm[(rho >> 1) * LDA + (j + K - 1)];
-      o1[(int64_t)(oi - sd.sup[0]) * sw + (oj - sd.sup[2])] = (rho & 1) ? z.y : z.x;
+    // the thread's column of the blocks: the tile column is fixed, a row adds
+    // a tile row's stride per 16 rows and a line of the tile per row
+    const int64_t tile_row = (int64_t)sd.gt[2] * sd.nfree * TILE_THREADS;
+    float* col = jbuf + sd.g_off + ((int64_t)(oj / TILE - sd.gt[1]) * sd.nfree + w.f) * TILE_THREADS + oj % TILE;
+    const float* sw = im.sw + oj;
+    const int r0 = sd.box[0] + w.by0, i0 = max(sd.sup[0] - r0, 0), i1 = min(sd.sup[1] - r0, B);
+    const float* z = reinterpret_cast<const float*>(sm + (j + K - 1));
+#pragma unroll 4
+    for (int i = i0 + threadIdx.x / N; i < i1; i += RSTEP) {
+      const int oi = r0 + i, rho = i + K - 1;
+      col[(oi / TILE - sd.gt[0]) * tile_row + (oi % TILE) * TILE] =
+          z[(rho >> 1) * (2 * LDA) + (rho & 1)] * sw[(int64_t)oi * im.W];
     }
   }
 }

@@ -1,86 +1,326 @@
 // J^T W J for the Levenberg-Marquardt step (Sec. "Optimization methods").
 //
 // J is never stored whole (the paper names its N_pixels x N_parameters memory
-// as LM's drawback): the convolved columns of each source are stored on that
-// source's support only, the others are its derivative images.
+// as LM's drawback): the columns of each source are stored on that source's
+// support only.
 //
-// Pass 1: each CTA owns one TILE x TILE image tile.  It loads sqrt(w)
-// dm/dtheta_k over the tile for every free slot of every source reaching the
-// tile into shared memory (pixel major), forms the tile's Gram matrix (3xTF32
-// tensor-core MMAs, or float64 on CUDA cores), and stores it, cut into the
-// blocks of its source pairs, into a scratch array where every source pair
-// keeps its tiles' blocks one after another (offsets planned on the host).
-// Pass 2: one warp per source pair adds its tiles' blocks in tile order and
+// Pass 1 forms the Gram matrix of every 16 x 16 image tile's free columns and
+// stores it, cut into the blocks of its source pairs, into a scratch array
+// where every source pair keeps its tiles' blocks one after another (offsets
+// planned on the host).  Pass 2 adds each pair's blocks in a fixed order and
 // writes each sum into the compressed-sparse-row J^T W J (and its mirror),
 // with plain stores where no other pair adds to the same entries (a shared
-// parameter, as in joint fits, makes float64 atomics necessary).  No
-// searches in the CSR and one write per entry instead of one atomic per tile.
+// parameter, as in joint fits, makes float64 atomics necessary).  No searches
+// in the CSR and one write per entry instead of one atomic per tile.
+//
+// Float path.  The columns come sqrt(w)-scaled in tile blocks (a column's 256
+// pixels of a tile in one kilobyte, zero outside the support), so a tile is
+// one bulk copy per column, without addresses, bounds or weights per pixel.
+// The products are 3xTF32 warp MMAs (m16n8k8; head x tail, tail x head, head
+// x head; the tail x tail term is below float32 rounding).  A warp holds the
+// accumulators of the whole upper triangle (up to 96 columns: 42 MMA tiles, 168
+// registers) and takes 64 of the tile's 256 pixels, so each value is read from
+// shared memory and split exactly once per tile, and the A and B fragments are
+// the same registers.  The four warps' 64-pixel float32 sums are joined by
+// compensated additions and kept as an unevaluated pair hi + lo of floats
+// (float64 conversions and additions for every entry of every tile would
+// occupy the thin float64 pipe longer than the MMAs take).  Bound by the
+// warp-MMA rate (a 48-column tile: 1152 MMAs, 2300 clocks of an SM at the
+// measured 303 TFLOP/s).  tcgen05 does not pay at these shapes: its M = 128 by
+// N = C MMA reads 4 + C/32 KB of operands from shared memory for
+// 128 x C x 8 products, so a 48-column tile takes some 1400 clocks of
+// shared-memory bandwidth for the MMAs and 1150 more to split and store both
+// halves of the operands -- no less than the warp MMAs; as built before (producer
+// warps gathering columns and storing swizzled heads and tails) it took 21 700
+// clocks per tile.  J^T W J of the 12 x 2048^2 joint fit (196 608 tiles, 38
+// columns on average) 14.2 -> 5.5 ms, of the 1536^2 crowded field 1.43 -> 0.65 ms,
+// of 64 cutouts 230 -> 80 us.
+//
+// Float64 path: one CTA per tile, columns gathered into shared memory, products
+// on the CUDA cores, float64 blocks.
 #include <algorithm>
+#include <type_traits>
 
 #include "ap_internal.cuh"
 
 namespace ap {
 
-template <typename T> struct GramCols { static constexpr int value = 160; };
-template <> struct GramCols<double> { static constexpr int value = 80; };
+// ---------------------------------------------------------------------------
+// float path, pass 1
+// ---------------------------------------------------------------------------
+namespace {
 
-template <typename T> struct Ld4;
-template <> struct Ld4<float> {
-  __device__ __forceinline__ static void ld(const float* p, float (&v)[4]) {
-    const float4 a = *reinterpret_cast<const float4*>(p);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+constexpr int GT_THREADS = 128;                 // four warps of 64 pixels
+constexpr uint32_t GT_WAIT_LIMIT = 1u << 16;    // mbarrier polls before giving up
+// Column pitch in shared memory: 32 bytes past a multiple of 128, so that the
+// eight columns x four pixel pairs of a fragment load (8 bytes a lane, half a
+// warp at a time) fall on 32 different banks.
+constexpr int GT_PITCH = TILE_THREADS * 4 + 32;       // whole tile (diagonal jobs)
+constexpr int GT_PITCH_H = TILE_THREADS * 2 + 32;     // half a tile (off-diagonal jobs)
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ uint32_t tf32_of(float x) {
+  uint32_t r;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+  return r;
+}
+
+__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
+  hi = tf32_of(x);
+  lo = tf32_of(x - __uint_as_float(hi));
+}
+
+__device__ __forceinline__ void mma_tf32(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                         uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+               "{%0,%1,%2,%3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const float* src, uint32_t bytes, uint32_t mbar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(mbar)
+               : "memory");
+}
+
+__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
+  for (uint32_t it = 0; it < GT_WAIT_LIMIT; ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred P1;\n\tmbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, P1;\n\t}\n"
+        : "=r"(done)
+        : "r"(mbar), "r"(parity)
+        : "memory");
+    if (done) return true;
   }
+  return false;
+}
+
+// one kind of fragment: 8 columns x 8 pixels, split; the lane's column is
+// `gid` of the group, its pixels 2 tig and 2 tig + 1 of the step (any
+// assignment of pixels to the MMA's k serves, as A and B take the same one)
+struct Frag {
+  uint32_t h0, h1, l0, l1;
 };
-template <> struct Ld4<double> {
-  __device__ __forceinline__ static void ld(const double* p, double (&v)[4]) {
-    const double2 a = *reinterpret_cast<const double2*>(p);
-    const double2 b = *reinterpret_cast<const double2*>(p + 2);
-    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+__device__ __forceinline__ void frag_load(Frag& f, const unsigned char* p) {
+  const float2 v = *reinterpret_cast<const float2*>(p);
+  split_tf32(v.x, f.h0, f.l0);
+  split_tf32(v.y, f.h1, f.l1);
+}
+
+// one 8-pixel step of NM x NN MMA tiles: A = column groups 2m, 2m + 1 of fa,
+// B = group n of fb; DIAG: only n >= 2m (the upper triangle).  The three
+// products go over all tiles in turn, so that consecutive MMAs are
+// independent; the small terms first.
+template <int NM, int NN, bool DIAG>
+__device__ __forceinline__ void mma_step(float (&d)[NM][NN][4], const Frag* fa, const Frag* fb) {
+#pragma unroll
+  for (int m = 0; m < NM; ++m)
+#pragma unroll
+    for (int n = DIAG ? 2 * m : 0; n < NN; ++n)
+      mma_tf32(d[m][n], fa[2 * m].h0, fa[2 * m + 1].h0, fa[2 * m].h1, fa[2 * m + 1].h1, fb[n].l0, fb[n].l1);
+#pragma unroll
+  for (int m = 0; m < NM; ++m)
+#pragma unroll
+    for (int n = DIAG ? 2 * m : 0; n < NN; ++n)
+      mma_tf32(d[m][n], fa[2 * m].l0, fa[2 * m + 1].l0, fa[2 * m].l1, fa[2 * m + 1].l1, fb[n].h0, fb[n].h1);
+#pragma unroll
+  for (int m = 0; m < NM; ++m)
+#pragma unroll
+    for (int n = DIAG ? 2 * m : 0; n < NN; ++n)
+      mma_tf32(d[m][n], fa[2 * m].h0, fa[2 * m + 1].h0, fa[2 * m].h1, fa[2 * m + 1].h1, fb[n].h0, fb[n].h1);
+}
+
+// Knuth's TwoSum: hi + lo carries the exact sum up to the rounding of lo
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
+  const float s = __fadd_rn(hi, x), bp = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(x, bp)));
+  hi = s;
+}
+
+template <int NM, int NN, bool DIAG>
+constexpr int gt_tiles() {
+  int t = 0;
+  for (int m = 0; m < NM; ++m) t += NN - (DIAG ? 2 * m : 0);
+  return t;
+}
+
+// The warps' sums in shared memory (where the columns were): row block m holds
+// its 16 rows over the columns right of the diagonal block, at a pitch of an
+// odd multiple of 8 floats -- the float2 stores of a fragment (8 rows x 4
+// pairs) and the row-wise loads are both free of bank conflicts.
+template <int NN, bool DIAG>
+__host__ __device__ constexpr int acc_pitch(int m) { return 8 * (NN - (DIAG ? 2 * m : 0)) + 8; }
+template <int NN, bool DIAG>
+__host__ __device__ constexpr int acc_block(int m) {
+  return DIAG ? 128 * ((NN + 1) * m - m * (m - 1)) : 16 * m * (8 * NN + 8);
+}
+template <int NM, int NN, bool DIAG>
+constexpr int gt_smem() {
+  const int cols = DIAG ? 16 * NM * GT_PITCH : (16 * NM + 8 * NN) * GT_PITCH_H;
+  const int acc = acc_block<NN, DIAG>(NM) * 4 * (GT_THREADS / 32);
+  return cols > acc ? cols : acc;
+}
+// CTAs per SM the registers are budgeted for (the accumulators and the
+// fragments live in registers: 4 per MMA tile and 4 per column group)
+template <int NM, int NN, bool DIAG>
+constexpr int gt_min_ctas() {
+  const int regs = 4 * gt_tiles<NM, NN, DIAG>() + 4 * (DIAG ? NN : 2 * NM + NN);
+  return regs > 120 ? 2 : regs > 80 ? 3 : regs > 56 ? 4 : 6;
+}
+
+constexpr int GT_STAGED_PAIRS = 256;   // pair offsets kept in shared memory (tiles of up to 22 sources)
+
+// One CTA per job: columns [ca0, ca0 + na) against [cb0, cb0 + nb) of a tile
+// (DIAG: the same columns, the upper triangle).
+template <int NM, int NN, bool DIAG>
+__global__ void __launch_bounds__(GT_THREADS, (gt_min_ctas<NM, NN, DIAG>())) gram_tile_kernel(
+    const GramJob* __restrict__ jobs, const GramEnt* __restrict__ ents, const float* __restrict__ cbuf,
+    const int64_t* __restrict__ tab_all, float2* __restrict__ scr, int* __restrict__ status) {
+  constexpr int NPH = DIAG ? 1 : 2;                          // loads of the tile's pixels
+  constexpr int PITCH = DIAG ? GT_PITCH : GT_PITCH_H;
+  constexpr uint32_t COLBYTES = TILE_THREADS * 4 / NPH;
+  constexpr int NW = GT_THREADS / 32;
+  constexpr int STEPS = TILE_THREADS / 8 / NW / NPH;         // 8-pixel steps of a warp per load
+  extern __shared__ __align__(128) unsigned char sm[];
+  __shared__ uint64_t mbar_store;
+  __shared__ int64_t s_tab[GT_STAGED_PAIRS];
+  __shared__ int s_ia[16 * NM], s_ib[DIAG ? 1 : 8 * NN];     // columns: (source << 8) | (free slot << 4) | free slots
+  const uint32_t mbar = smem_u32(&mbar_store);
+  const GramJob job = jobs[blockIdx.x];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int gid = lane >> 2, tig = lane & 3;
+  const int L = job.L;
+  const int64_t* tab = tab_all + job.tab0;
+  const bool staged = L * (L + 1) / 2 <= GT_STAGED_PAIRS;
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-};
-
-// Row stride of the pixel-major column blocks: for the tensor-core path a
-// multiple of 32 plus 8 floats, so the eight rows x four lanes of a fragment
-// load hit 32 different banks; cb + 4 for the float64 path.
-template <typename T>
-__host__ __device__ constexpr int gram_stride(int cb) {
-  return sizeof(T) == 4 ? ((cb + 31) / 32) * 32 + 8 : cb + 4;
+  float d[NM][NN][4];
+#pragma unroll
+  for (int m = 0; m < NM; ++m)
+#pragma unroll
+    for (int n = 0; n < NN; ++n)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) d[m][n][q] = 0.f;
+#pragma unroll 1
+  for (int ph = 0; ph < NPH; ++ph) {
+    if (tid == 0) {
+      const uint32_t bytes = (uint32_t)(job.na + (DIAG ? 0 : job.nb)) * COLBYTES;
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
+    }
+    __syncthreads();   // the expected bytes are set (and the last load's columns read)
+    for (int x = tid; x < L; x += GT_THREADS) {
+      const GramEnt e = ents[job.e0 + x];
+      const float* src = cbuf + e.off + ph * (TILE_THREADS / NPH);
+      for (int f = 0; f < e.nf; ++f) {
+        const int a = e.col0 + f - job.ca0, b = e.col0 + f - job.cb0;
+        if (a >= 0 && a < job.na) {
+          bulk_load(smem_u32(sm + a * PITCH), src + f * TILE_THREADS, COLBYTES, mbar);
+          s_ia[a] = (x << 8) | (f << 4) | e.nf;
+        }
+        if (!DIAG && b >= 0 && b < job.nb) {
+          bulk_load(smem_u32(sm + (16 * NM + b) * PITCH), src + f * TILE_THREADS, COLBYTES, mbar);
+          s_ib[b] = (x << 8) | (f << 4) | e.nf;
+        }
+      }
+    }
+    if (ph == 0 && staged)
+      for (int p = tid; p < L * (L + 1) / 2; p += GT_THREADS) s_tab[p] = tab[p];
+    if (!__syncthreads_and(mbar_wait(mbar, ph & 1))) {
+      // the copies did not arrive within the limit: one more wait, so that
+      // none is in flight when the CTA leaves
+      if (tid == 0) atomicCAS(status, 0, AP_ERR_TIMEOUT);
+      mbar_wait(mbar, ph & 1);
+      return;
+    }
+    const unsigned char* base = sm + gid * PITCH + tig * 8 + warp * STEPS * 32;
+#pragma unroll(gt_tiles<NM, NN, DIAG>() <= 12 ? 2 : 1)
+    for (int s = 0; s < STEPS; ++s) {
+      Frag fa[DIAG ? NN : 2 * NM], fb[DIAG ? 1 : NN];
+#pragma unroll
+      for (int g = 0; g < (DIAG ? NN : 2 * NM); ++g) frag_load(fa[g], base + g * 8 * PITCH + s * 32);
+      if constexpr (!DIAG) {
+#pragma unroll
+        for (int g = 0; g < NN; ++g) frag_load(fb[g], base + (16 * NM + g * 8) * PITCH + s * 32);
+      }
+      mma_step<NM, NN, DIAG>(d, fa, DIAG ? fa : fb);
+    }
+    __syncthreads();   // every warp has read the columns
+  }
+  constexpr int ACC = acc_block<NN, DIAG>(NM);
+  float* acc = reinterpret_cast<float*>(sm);
+#pragma unroll
+  for (int m = 0; m < NM; ++m) {
+    float* mine = acc + warp * ACC + acc_block<NN, DIAG>(m) + gid * acc_pitch<NN, DIAG>(m) + 2 * tig;
+#pragma unroll
+    for (int n = DIAG ? 2 * m : 0; n < NN; ++n) {
+      float* q = mine + 8 * (n - (DIAG ? 2 * m : 0));
+      *reinterpret_cast<float2*>(q) = make_float2(d[m][n][0], d[m][n][1]);
+      *reinterpret_cast<float2*>(q + 8 * acc_pitch<NN, DIAG>(m)) = make_float2(d[m][n][2], d[m][n][3]);
+    }
+  }
+  __syncthreads();
+  // the source pairs' blocks: a warp takes every fourth row, its lanes the
+  // row's columns (a run of a source's columns is a run of its pair's block)
+  const int* ib_of = DIAG ? s_ia : s_ib;
+#pragma unroll 1
+  for (int c0 = 0; c0 < job.nb; c0 += 32) {
+    const int cb = c0 + lane;
+    const int ib = cb < job.nb ? ib_of[cb] : 0;
+    const int b = ib >> 8, fb = (ib >> 4) & 15, mb = ib & 15;
+    const int rows = DIAG ? min(job.na, c0 + 32) : job.na;
+#pragma unroll 2
+    for (int ca = warp; ca < rows; ca += NW) {
+      const int ia = s_ia[ca], a = ia >> 8, fa = (ia >> 4) & 15, m = ca >> 4;
+      if (cb < job.nb && (!DIAG || cb >= ca)) {
+        const float* v =
+            acc + acc_block<NN, DIAG>(m) + (ca & 15) * acc_pitch<NN, DIAG>(m) + cb - (DIAG ? 16 * m : 0);
+        // the four 64-pixel sums as hi + lo
+        float h0 = v[0], l0 = 0.f, h1 = v[2 * ACC], l1 = 0.f;
+        two_sum(h0, l0, v[ACC]);
+        two_sum(h1, l1, v[3 * ACC]);
+        two_sum(h0, l0, h1);
+        const int p = a * L - (a * (a - 1)) / 2 + (b - a);
+        scr[(staged ? s_tab[p] : tab[p]) + fa * mb + fb] = make_float2(h0, __fadd_rn(l0, l1));
+      }
+    }
+  }
 }
 
-// Column position of element (pixel p, column c) in its pixel row.  Float
-// path: c XOR ((p / 4) mod 8), which keeps c in its aligned group of 8 and
-// makes both access patterns conflict-free with the stride above (= 8 mod
-// 32): the row writes (32 pixels, one column) and the MMA fragment loads (4
-// pixels x 8 columns).  Float64 path: unswizzled (4-column vector loads).
-template <typename T>
-__device__ __forceinline__ int gram_swz(int p, int c) {
-  return sizeof(T) == 4 ? (c ^ ((p >> 2) & 7)) : c;
+template <int NM, int NN, bool DIAG>
+void gt_launch(const GramJob* jobs, int n, const GramPlan& gp, const float* cbuf, int* status, cudaStream_t st) {
+  gram_tile_kernel<NM, NN, DIAG><<<n, GT_THREADS, gt_smem<NM, NN, DIAG>(), st>>>(
+      jobs, gp.ents, cbuf, gp.tab, reinterpret_cast<float2*>(gp.scr), status);
 }
 
-// Asynchronous copy of one element global -> shared (cp.async, sm_80+): the
-// copies of all of a thread's columns are in flight together.
-template <typename T>
-__device__ __forceinline__ void cp_async_elem(T* dst_smem, const T* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
-  if constexpr (sizeof(T) == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
-}
+}  // namespace
 
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// ---------------------------------------------------------------------------
+// float64 path, pass 1
+// ---------------------------------------------------------------------------
+constexpr int GRAM64_CB = 32;   // columns of a block
+
+__device__ __forceinline__ void ld4(const double* p, double (&v)[4]) {
+  const double2 a = *reinterpret_cast<const double2*>(p);
+  const double2 b = *reinterpret_cast<const double2*>(p + 2);
+  v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
 
 // Load columns [c0, c0 + cb) of the tile (in (source, slot) order) into a
 // pixel-major block of row stride CP, scaled by sqrt(w) of the thread's
 // pixel; returns the number loaded.  Every thread fills its own row: copies
-// are issued for all its in-box values, then awaited, then scaled.
-template <typename T>
-__device__ __forceinline__ int load_columns(T* blk, int CP, int c0, int cb, const TileWork& w,
+// (cp.async, all in flight together) are issued for its in-box values, then
+// awaited, then scaled.
+__device__ __forceinline__ int load_columns(double* blk, int CP, int c0, int cb, const TileWork& w,
                                             const int* __restrict__ jt_src, const SourceDev* __restrict__ srcs,
-                                            const T* __restrict__ dbuf, const T* __restrict__ jbuf, int i, int j,
-                                            bool inside, T sw, int* colp) {
-  T* myrow = blk + threadIdx.x * CP;
-  const int p = threadIdx.x;
+                                            const double* __restrict__ dbuf, const double* __restrict__ jbuf, int i,
+                                            int j, bool inside, double sw, int* colp) {
+  double* myrow = blk + threadIdx.x * CP;
   int col = 0, n = 0;
   for (int e = w.e0; e < w.e1 && n < cb; ++e) {
     const SourceDev& sd = srcs[jt_src[e]];
@@ -92,14 +332,18 @@ __device__ __forceinline__ int load_columns(T* blk, int CP, int c0, int cb, cons
     const bool in_b = inside && i >= bx[0] && i < bx[1] && j >= bx[2] && j < bx[3];
     const int bw = bx[3] - bx[2];
     const int64_t area = (int64_t)(bx[1] - bx[0]) * bw;
-    const T* base = (sd.conv ? jbuf + sd.j_off : dbuf + sd.d_off) + (in_b ? (int64_t)(i - bx[0]) * bw + (j - bx[2]) : 0);
+    const double* base =
+        (sd.conv ? jbuf + sd.j_off : dbuf + sd.d_off) + (in_b ? (int64_t)(i - bx[0]) * bw + (j - bx[2]) : 0);
     int f = 0;
 #pragma unroll
     for (int k = 0; k < MAX_SLOTS; ++k) {
       if (k >= sd.nslot || sd.pidx[k] < 0) continue;
       if (col >= c0 && n < cb) {
-        if (in_b) cp_async_elem(myrow + gram_swz<T>(p, n), base + k * area);
-        else myrow[gram_swz<T>(p, n)] = (T)0;
+        if (in_b)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(myrow + n)), "l"(base + k * area)
+                       : "memory");
+        else
+          myrow[n] = 0.0;
         // column info: local source index, free-slot index, free columns of the source
         if (threadIdx.x == 0) colp[n] = ((e - w.e0) << 8) | (f << 4) | nfree;
         ++n;
@@ -108,29 +352,17 @@ __device__ __forceinline__ int load_columns(T* blk, int CP, int c0, int cb, cons
       ++col;
     }
   }
-  for (int c = n; c < ((n + 15) & ~15) && c < CP; ++c) myrow[gram_swz<T>(p, c)] = (T)0;
-  cp_async_wait_all();
-  for (int c = 0; c < n; ++c) myrow[gram_swz<T>(p, c)] *= sw;
+  for (int c = n; c < ((n + 15) & ~15) && c < CP; ++c) myrow[c] = 0.0;
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  for (int c = 0; c < n; ++c) myrow[c] *= sw;
   return n;
 }
 
-// Store one tile Gram entry (columns ca <= cb with column infos ia, ib) into
-// its source pair's block: pairs of the L tile sources are numbered
-// row-major over a <= b.
-__device__ __forceinline__ void gram_store(double g, int ia, int ib, int L, const int64_t* __restrict__ tab,
-                                           const int* __restrict__ tabs, double* __restrict__ scr) {
-  const int la = ia >> 8, fa = (ia >> 4) & 15;
-  const int lb = ib >> 8, fb = (ib >> 4) & 15, mb = ib & 15;
-  const int pidx = la * L - (la * (la - 1)) / 2 + (lb - la);
-  scr[tab[pidx] + (int64_t)(fa * mb + fb) * tabs[pidx]] = g;
-}
-
 // Gram of column block A (na columns) with column block B (nb_ columns) of
-// the tile, stored into the pair blocks; diag = the blocks are the same.
-template <typename T>
-__device__ void gram_pair(const T* ja, const T* jb, int CP, int na, int nbc, bool diag, const int* colpa,
-                          const int* colpb, int L, const int64_t* __restrict__ tab, const int* __restrict__ tabs,
-                          double* __restrict__ scr) {
+// the tile, stored into the pair blocks (pairs of the L tile sources are
+// numbered row-major over a <= b); diag = the blocks are the same.
+__device__ void gram_pair(const double* ja, const double* jb, int CP, int na, int nbc, bool diag, const int* colpa,
+                          const int* colpb, int L, const int64_t* __restrict__ tab, double* __restrict__ scr) {
   const int tid = threadIdx.x;
   const int ba = (na + 3) >> 2, bb = (nbc + 3) >> 2;   // 4-column sub-blocks
   const int npb = diag ? ba * (ba + 1) / 2 : ba * bb;
@@ -153,35 +385,29 @@ __device__ void gram_pair(const T* ja, const T* jb, int CP, int na, int nbc, boo
       A = pb / bb;
       B = pb - A * bb;
     }
-    T acc[4][4];
+    double acc[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = (T)0;
+      for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
     if (active) {
-      const T* pa = ja + 4 * A;
-      const T* pbp = jb + 4 * B;
+      const double* pa = ja + 4 * A;
+      const double* pbp = jb + 4 * B;
       for (int t = seg * seglen; t < (seg + 1) * seglen; ++t) {
-        T va[4], vb[4];
-        Ld4<T>::ld(pa + t * CP, va);
-        Ld4<T>::ld(pbp + t * CP, vb);
+        double va[4], vb[4];
+        ld4(pa + t * CP, va);
+        ld4(pbp + t * CP, vb);
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
           for (int b = 0; b < 4; ++b) acc[a][b] += va[a] * vb[b];
       }
     }
-    // segment partial sums (at most 64 pixels each in T) combine in float64
-    double accd[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) accd[a][b] = (double)acc[a][b];
     for (int o = NS >> 1; o > 0; o >>= 1)
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) accd[a][b] += __shfl_xor_sync(0xffffffffu, accd[a][b], o);
+        for (int b = 0; b < 4; ++b) acc[a][b] += __shfl_xor_sync(0xffffffffu, acc[a][b], o);
     if (!active || seg != 0) continue;
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
@@ -189,122 +415,26 @@ __device__ void gram_pair(const T* ja, const T* jb, int CP, int na, int nbc, boo
       for (int b = 0; b < 4; ++b) {
         const int ca = 4 * A + a, cb = 4 * B + b;
         if (ca >= na || cb >= nbc || (diag && cb < ca)) continue;
-        gram_store(accd[a][b], colpa[ca], colpb[cb], L, tab, tabs, scr);
+        const int ia = colpa[ca], ib = colpb[cb];
+        const int la = ia >> 8, fa = (ia >> 4) & 15, lb = ib >> 8, fb = (ib >> 4) & 15, mb = ib & 15;
+        scr[tab[la * L - (la * (la - 1)) / 2 + (lb - la)] + fa * mb + fb] = acc[a][b];
       }
     }
   }
-}
-
-// ---------------------------------------------------------------------------
-// 3xTF32 tensor-core Gram (float path).  Each warp owns 16 x 8 output tiles
-// of the block pair; for 8 pixels at a time it loads the A fragment (16
-// columns of block A) and the B fragment (8 columns of block B) from the
-// pixel-major shared blocks, splits every value into a TF32 head and a TF32
-// tail, and issues three m16n8k8 MMAs (head*head + head*tail + tail*head,
-// the tail*tail term is below float32 rounding).  Products accumulate in
-// float32 over 64 pixels, then join a float64 sum.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t tf32_of(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return r;
-}
-
-__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
-  hi = tf32_of(x);
-  lo = tf32_of(x - __uint_as_float(hi));
-}
-
-__device__ __forceinline__ void mma_tf32(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                         uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-               "{%0,%1,%2,%3};"
-               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-__device__ void gram_pair_tc(const float* ja, const float* jb, int CP, int na, int nbc, bool diag, const int* colpa,
-                             const int* colpb, int L, const int64_t* __restrict__ tab, const int* __restrict__ tabs,
-                          double* __restrict__ scr) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gid = lane >> 2, tig = lane & 3;
-  const int mt_n = (na + 15) >> 4, nt_n = (nbc + 7) >> 3;
-  for (int t = warp; t < mt_n * nt_n; t += TILE_THREADS / 32) {
-    const int mt = t / nt_n, nt = t - mt * nt_n;
-    const int m0 = 16 * mt, n0 = 8 * nt;
-    if (diag && n0 + 8 <= m0) continue;   // entirely below the diagonal: its mirror is computed
-    // 64-pixel float32 segments joined by a compensated float32 sum
-    // (Knuth's TwoSum: hi + lo carries the exact sum of the segments up to
-    // the rounding of lo), converted to float64 once per output
-    float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int seg = 0; seg < TILE_THREADS; seg += 64) {
-      float d[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 2
-      for (int k0 = seg; k0 < seg + 64; k0 += 8) {
-        // pixels p0 (fragment rows 0-3) and p0 + 4 (rows 4-7), swizzled columns
-        const int p0 = k0 + tig, p1 = p0 + 4;
-        const int s0 = (p0 >> 2) & 7, s1 = (p1 >> 2) & 7;
-        const float* r0 = ja + p0 * CP;
-        const float* r1 = ja + p1 * CP;
-        uint32_t ah0, al0, ah1, al1, ah2, al2, ah3, al3, bh0, bl0, bh1, bl1;
-        split_tf32(r0[m0 + (gid ^ s0)], ah0, al0);
-        split_tf32(r0[m0 + 8 + (gid ^ s0)], ah1, al1);
-        split_tf32(r1[m0 + (gid ^ s1)], ah2, al2);
-        split_tf32(r1[m0 + 8 + (gid ^ s1)], ah3, al3);
-        split_tf32(jb[p0 * CP + n0 + (gid ^ s0)], bh0, bl0);
-        split_tf32(jb[p1 * CP + n0 + (gid ^ s1)], bh1, bl1);
-        mma_tf32(d, ah0, ah1, ah2, ah3, bl0, bl1);
-        mma_tf32(d, al0, al1, al2, al3, bh0, bh1);
-        mma_tf32(d, ah0, ah1, ah2, ah3, bh0, bh1);
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float sum = __fadd_rn(hi[q], d[q]);
-        const float bp = __fsub_rn(sum, hi[q]);
-        const float err = __fadd_rn(__fsub_rn(hi[q], __fsub_rn(sum, bp)), __fsub_rn(d[q], bp));
-        hi[q] = sum;
-        lo[q] = __fadd_rn(lo[q], err);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int ca = m0 + gid + (q >> 1) * 8;
-      const int cb = n0 + 2 * tig + (q & 1);
-      if (ca >= na || cb >= nbc || (diag && cb < ca)) continue;
-      gram_store((double)hi[q] + (double)lo[q], colpa[ca], colpb[cb], L, tab, tabs, scr);
-    }
-  }
-}
-
-template <typename T>
-__device__ __forceinline__ void gram_pair_any(const T* ja, const T* jb, int CP, int na, int nbc, bool diag,
-                                              const int* colpa, const int* colpb, int L, const int64_t* tab,
-                                              const int* tabs, double* scr) {
-  if constexpr (sizeof(T) == 4)
-    gram_pair_tc(reinterpret_cast<const float*>(ja), reinterpret_cast<const float*>(jb), CP, na, nbc, diag, colpa,
-                 colpb, L, tab, tabs, scr);
-  else
-    gram_pair<T>(ja, jb, CP, na, nbc, diag, colpa, colpb, L, tab, tabs, scr);
 }
 
 // One CTA per image tile.  The tile's C columns are processed in blocks of
 // cb: block I is loaded once, then paired with every block J >= I (the Gram
 // is symmetric), so any number of columns fits in two shared blocks.
-template <typename T>
-__global__ void __launch_bounds__(TILE_THREADS) gram_kernel(const TileWork* __restrict__ work,
-                                                            const int* __restrict__ jt_src,
-                                                            const SourceDev* __restrict__ srcs,
-                                                            const ImageDev* __restrict__ imgs,
-                                                            const T* __restrict__ dbuf, const T* __restrict__ jbuf,
-                                                            const int64_t* __restrict__ tab0,
-                                                            const int64_t* __restrict__ tab_all,
-                                                            const int* __restrict__ tabs_all,
-                                                            double* __restrict__ scr, int t_first, int cb,
-                                                            int two_blocks, int* __restrict__ status) {
-  const int CP = gram_stride<T>(cb);
+__global__ void __launch_bounds__(TILE_THREADS) gram_f64_kernel(
+    const TileWork* __restrict__ work, const int* __restrict__ jt_src, const SourceDev* __restrict__ srcs,
+    const ImageDev* __restrict__ imgs, const double* __restrict__ dbuf, const double* __restrict__ jbuf,
+    const int64_t* __restrict__ tab0, const int64_t* __restrict__ tab_all, double* __restrict__ scr, int t_first,
+    int cb, int two_blocks) {
+  const int CP = cb + 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* blk0 = reinterpret_cast<T*>(smem_raw);
-  T* blk1 = blk0 + TILE_THREADS * CP;
+  double* blk0 = reinterpret_cast<double*>(smem_raw);
+  double* blk1 = blk0 + TILE_THREADS * CP;
   int* colp0 = reinterpret_cast<int*>(blk0 + (two_blocks ? 2 : 1) * TILE_THREADS * CP);
   int* colp1 = colp0 + CP;
   const int tile = t_first + blockIdx.x;
@@ -313,14 +443,11 @@ __global__ void __launch_bounds__(TILE_THREADS) gram_kernel(const TileWork* __re
   const int tid = threadIdx.x;
   const int i = w.r0 + tid / TILE, j = w.c0 + tid % TILE;
   const bool inside = i < im.H && j < im.W;
-  T sw = (T)0;
+  double sw = 0.0;
   if (inside) {
     const size_t o = (size_t)i * im.W + j;
     const float var = im.var[o];
-    // sqrt(w) in the column type: float32 (correctly rounded division and
-    // root) in the mixed form, float64 in the float64 form
-    if ((im.mask == nullptr || im.mask[o] == 0) && var > 0.f && isfinite(var))
-      sw = sizeof(T) == 4 ? (T)(1.0f / sqrtf(var)) : (T)sqrt(1.0 / (double)var);
+    if ((im.mask == nullptr || im.mask[o] == 0) && var > 0.f && isfinite(var)) sw = sqrt(1.0 / (double)var);
   }
   // total free columns of the tile
   int C = 0;
@@ -329,31 +456,75 @@ __global__ void __launch_bounds__(TILE_THREADS) gram_kernel(const TileWork* __re
     for (int k = 0; k < sd.nslot; ++k) C += sd.pidx[k] >= 0;
   }
   const int nblk = (C + cb - 1) / cb;
-  if (nblk > 1 && !two_blocks) {
-    if (tid == 0) atomicCAS(status, 0, AP_ERR_ARG);
-    return;
-  }
   const int L = w.e1 - w.e0;
   const int64_t* tab = tab_all + tab0[tile];
-  const int* tabs = tabs_all + tab0[tile];
   for (int I = 0; I < nblk; ++I) {
     __syncthreads();
-    const int na = load_columns<T>(blk0, CP, I * cb, cb, w, jt_src, srcs, dbuf, jbuf, i, j, inside, sw, colp0);
+    const int na = load_columns(blk0, CP, I * cb, cb, w, jt_src, srcs, dbuf, jbuf, i, j, inside, sw, colp0);
     __syncthreads();
-    gram_pair_any<T>(blk0, blk0, CP, na, na, true, colp0, colp0, L, tab, tabs, scr);
+    gram_pair(blk0, blk0, CP, na, na, true, colp0, colp0, L, tab, scr);
     for (int J = I + 1; J < nblk; ++J) {
       __syncthreads();
-      const int nb_ = load_columns<T>(blk1, CP, J * cb, cb, w, jt_src, srcs, dbuf, jbuf, i, j, inside, sw, colp1);
+      const int nb_ = load_columns(blk1, CP, J * cb, cb, w, jt_src, srcs, dbuf, jbuf, i, j, inside, sw, colp1);
       __syncthreads();
-      gram_pair_any<T>(blk0, blk1, CP, na, nb_, false, colp0, colp1, L, tab, tabs, scr);
+      gram_pair(blk0, blk1, CP, na, nb_, false, colp0, colp1, L, tab, scr);
     }
   }
 }
 
-// Pass 2, light pairs: one warp per pair; lane e adds entry e of the pair's
-// block over its tiles in tile order (float64) and writes it and its mirror.
-__device__ __forceinline__ void gram_write(const GramPair& gp, int64_t pab, int64_t pba, double s,
+static size_t gram64_smem(int cb, int two) {
+  const int CP = cb + 4;
+  return (size_t)(two ? 2 : 1) * TILE_THREADS * CP * sizeof(double) + (size_t)2 * CP * sizeof(int);
+}
+
+// ---------------------------------------------------------------------------
+// pass 2: the pairs' sums over their tiles.  A pair's blocks lie one after
+// another (entry fastest), so consecutive threads read consecutive values:
+// thread t takes entry t mod ne of tiles t / ne, t / ne + T, ...  Each thread
+// sums hi + lo compensated (float path) or in float64, the threads of an entry
+// are joined in float64 in a fixed order (deterministic).
+// ---------------------------------------------------------------------------
+template <typename V> struct TileSum;
+template <> struct TileSum<float2> {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float2 v) {
+    two_sum(hi, lo, v.x);
+    lo = __fadd_rn(lo, v.y);
+  }
+  __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
+};
+template <> struct TileSum<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ double get() const { return s; }
+};
+
+// entry values src[k ne], k = k0, k0 + step, ... below cnt: eight loads in flight
+template <typename V>
+__device__ __forceinline__ double tile_sum(const V* __restrict__ src, int ne, int k0, int step, int cnt) {
+  TileSum<V> acc;
+  int k = k0;
+  for (; k + 7 * step < cnt; k += 8 * step) {
+    V v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = src[(int64_t)(k + u * step) * ne];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) acc.add(v[u]);
+  }
+  V v[8];
+#pragma unroll
+  for (int u = 0; u < 7; ++u)
+    if (k + u * step < cnt) v[u] = src[(int64_t)(k + u * step) * ne];
+#pragma unroll
+  for (int u = 0; u < 7; ++u)
+    if (k + u * step < cnt) acc.add(v[u]);
+  return acc.get();
+}
+
+__device__ __forceinline__ void gram_write(const GramPair& gp, const int64_t* __restrict__ pos, int e, double s,
                                            double* __restrict__ vals) {
+  const int64_t pab = pos[gp.pos + 2 * e], pba = pos[gp.pos + 2 * e + 1];
+  if (pab < 0) return;   // below the diagonal of a source's own block
   if (gp.excl) {
     vals[pab] = s;
     if (pba >= 0) vals[pba] = s;
@@ -363,183 +534,177 @@ __device__ __forceinline__ void gram_write(const GramPair& gp, int64_t pab, int6
   }
 }
 
+// pairs of few values (n_light of them, first in the list): a warp each
+template <typename V>
 __global__ void __launch_bounds__(256) gram_reduce_kernel(const GramPair* __restrict__ pairs, int n_pairs,
-                                                          const int64_t* __restrict__ pos,
-                                                          const double* __restrict__ scr,
+                                                          const int64_t* __restrict__ pos, const V* __restrict__ scr,
                                                           double* __restrict__ vals) {
   const int lane = threadIdx.x & 31;
   const int w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
   for (int p = w0; p < n_pairs; p += nw) {
     const GramPair gp = pairs[p];
     const int ne = gp.ma * gp.mb;
-    for (int e = lane; e < ne; e += 32) {
-      const int64_t pab = pos[gp.pos + 2 * e], pba = pos[gp.pos + 2 * e + 1];
-      if (pab < 0) continue;   // below the diagonal of a source's own block
-      const double* src = scr + gp.base + e;
-      double acc[4] = {0.0, 0.0, 0.0, 0.0};
-      int k = 0;
-      for (; k + 3 < gp.cnt; k += 4) {   // four independent loads in flight
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u] += src[(int64_t)(k + u) * ne];
-      }
-      double tail = 0.0;
-      for (; k < gp.cnt; ++k) tail += src[(int64_t)k * ne];
-      gram_write(gp, pab, pba, ((acc[0] + acc[1]) + (acc[2] + acc[3])) + tail, vals);
+    const V* src = scr + gp.base;
+    if (ne > 16) {   // one tile at a time, an entry (or two) per lane
+      for (int e = lane; e < ne; e += 32) gram_write(gp, pos, e, tile_sum(src + e, ne, 0, 1, gp.cnt), vals);
+    } else {         // 32 / ne tiles side by side
+      const int T = 32 / ne, e = lane % ne, t = lane / ne;
+      const double part = t < T ? tile_sum(src + e, ne, t, T, gp.cnt) : 0.0;
+      double s = 0.0;
+      for (int k = 0; k < T; ++k) s += __shfl_sync(0xffffffffu, part, (k * ne + e) & 31);
+      if (lane < ne) gram_write(gp, pos, e, s, vals);
     }
   }
 }
 
-// Pass 2, heavy pairs, entries spanning many tiles (a source and the sky,
-// the sky and itself): one CTA per entry from a planned work list; the
-// entry's tiles are contiguous, the threads stride over them and a fixed
-// tree joins the partials (deterministic).
-__global__ void __launch_bounds__(256) gram_reduce_heavy_kernel(const GramPair* __restrict__ pairs,
-                                                                const int* __restrict__ items,
-                                                                const int64_t* __restrict__ pos,
-                                                                const double* __restrict__ scr,
-                                                                double* __restrict__ vals) {
-  __shared__ double red[8];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int item = items[blockIdx.x];
-  const GramPair gp = pairs[item >> 6];
-  const int e = item & 63;
-  const int64_t pab = pos[gp.pos + 2 * e], pba = pos[gp.pos + 2 * e + 1];
-  const double* src = scr + gp.base + (int64_t)e * gp.cnt;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  int k = threadIdx.x;
-  for (; k + 768 < gp.cnt; k += 1024) {
-#pragma unroll
-    for (int u = 0; u < 4; ++u) acc[u] += src[k + 256 * u];
-  }
-  double tail = 0.0;
-  for (; k < gp.cnt; k += 256) tail += src[k];
-  double s = ((acc[0] + acc[1]) + (acc[2] + acc[3])) + tail;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) red[warp] = s;
+// the other pairs: a CTA per run of up to GRAM_RUN_TILES tiles; the CTA that
+// finishes a pair last adds its runs in order
+template <typename V>
+__global__ void __launch_bounds__(256) gram_reduce_run_kernel(const GramPair* __restrict__ pairs,
+                                                              const GramRun* __restrict__ runs,
+                                                              const int64_t* __restrict__ pos,
+                                                              const V* __restrict__ scr, double* __restrict__ part,
+                                                              int* __restrict__ done, double* __restrict__ vals) {
+  __shared__ double red[256];
+  __shared__ int last;
+  const GramRun rn = runs[blockIdx.x];
+  const GramPair gp = pairs[rn.pair];
+  const int ne = gp.ma * gp.mb, T = 256 / ne;
+  const int e = threadIdx.x % ne, t = threadIdx.x / ne;
+  if (t < T) red[threadIdx.x] = tile_sum(scr + gp.base + e, ne, rn.k0 + t, T, rn.k1);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    gram_write(gp, pab, pba, t, vals);
+  double s = 0.0;
+  if ((int)threadIdx.x < ne) {
+    for (int k = 0; k < T; ++k) s += red[k * ne + threadIdx.x];
+    if (rn.n_runs == 1)
+      gram_write(gp, pos, threadIdx.x, s, vals);
+    else
+      part[(int64_t)(rn.first + rn.run) * 64 + threadIdx.x] = s;
   }
+  if (rn.n_runs == 1) return;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&done[rn.first], 1) == rn.n_runs - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if ((int)threadIdx.x < ne) {
+    s = 0.0;
+    for (int k = 0; k < rn.n_runs; ++k) s += __ldcg(part + (int64_t)(rn.first + k) * 64 + threadIdx.x);
+    gram_write(gp, pos, threadIdx.x, s, vals);
+  }
+  if (threadIdx.x == 0) done[rn.first] = 0;   // ready for the next call
 }
 
-// Pass 2, heavy pairs, the other entries (up to GRAM_CTA_TILES tiles): one
-// warp per entry, grid-stride over the work list; lane l adds tiles l,
-// l + 32, ... in four independent chains and a fixed shuffle tree joins the
-// lanes (deterministic).
-__global__ void __launch_bounds__(256) gram_reduce_heavy_warp_kernel(const GramPair* __restrict__ pairs,
-                                                                     const int* __restrict__ items, int n_items,
-                                                                     const int64_t* __restrict__ pos,
-                                                                     const double* __restrict__ scr,
-                                                                     double* __restrict__ vals) {
-  const int lane = threadIdx.x & 31;
-  const int w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-  for (int it = w0; it < n_items; it += nw) {
-    const int item = items[it];
-    const GramPair gp = pairs[item >> 6];
-    const int e = item & 63;
-    const double* src = scr + gp.base + (int64_t)e * gp.cnt;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    int k = lane;
-    for (; k + 96 < gp.cnt; k += 128) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) acc[u] += src[k + 32 * u];
+// ---------------------------------------------------------------------------
+// jobs and launches
+// ---------------------------------------------------------------------------
+void gram64_blocking(int maxc, int* cb, int* two) {
+  const int m = ((maxc < 4 ? 4 : maxc) + 3) & ~3;
+  *cb = m < GRAM64_CB ? m : GRAM64_CB;
+  *two = m > GRAM64_CB;
+}
+
+// The jobs of the tiles' column counts, grouped by kernel form: form g = 1..6
+// takes up to 16 g columns (the triangle's accumulators fit the registers up
+// to 96); a tile past 96 columns is cut into blocks of 64, a diagonal job each
+// and an off-diagonal job (form 7, 64 x 64) for every two.
+void gram_plan_jobs(const std::vector<TileWork>& tiles, const std::vector<int64_t>& tab0,
+                    const std::vector<int>& tile_ncol, std::vector<GramJob>& jobs, std::vector<GramRange>& ranges) {
+  std::vector<GramJob> by[GRAM_FORMS + 1];
+  for (int t = 0; t < (int)tile_ncol.size(); ++t) {
+    const int C = tile_ncol[t];
+    if (C <= 0) continue;
+    const int e0 = tiles[t].e0, L = tiles[t].e1 - e0;
+    if (C <= 96) {
+      by[(C + 15) / 16].push_back(GramJob{tab0[t], e0, L, 0, C, 0, C});
+      continue;
     }
-    double tail = 0.0;
-    for (; k < gp.cnt; k += 32) tail += src[k];
-    double s = ((acc[0] + acc[1]) + (acc[2] + acc[3])) + tail;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) gram_write(gp, pos[gp.pos + 2 * e], pos[gp.pos + 2 * e + 1], s, vals);
+    for (int a = 0; a < C; a += 64) {
+      const int na = std::min(64, C - a);
+      by[(na + 15) / 16].push_back(GramJob{tab0[t], e0, L, a, na, a, na});
+      for (int b = a + 64; b < C; b += 64)
+        by[GRAM_FORMS].push_back(GramJob{tab0[t], e0, L, a, na, b, std::min(64, C - b)});
+    }
+  }
+  for (int f = GRAM_FORMS; f >= 1; --f) {   // the longest jobs first
+    if (by[f].empty()) continue;
+    ranges.push_back(GramRange{(int)jobs.size(), (int)(jobs.size() + by[f].size()), f, 0});
+    jobs.insert(jobs.end(), by[f].begin(), by[f].end());
   }
 }
 
-template <typename T>
-size_t gram_smem_bytes(int cb, int two) {
-  const int CP = gram_stride<T>(cb);
-  return (size_t)(two ? 2 : 1) * TILE_THREADS * CP * sizeof(T) + (size_t)2 * CP * sizeof(int);
-}
-
-int gram_max_cols(int is_double) { return is_double ? GramCols<double>::value : GramCols<float>::value; }
-
-// Column block size of a problem: the largest column count of any tile,
-// rounded to 16 (float) / 4 (double), capped at 96 (float: one block in about
-// 100 KB of shared memory) / 32 (double); two blocks only when some tile needs
-// them.
-template <typename T>
-void gram_blocking(int maxc, int* cb, int* two) {
-  const int cap = sizeof(T) == 4 ? 96 : 32;
-  const int m = sizeof(T) == 4 ? ((maxc < 16 ? 16 : maxc) + 15) & ~15 : ((maxc < 4 ? 4 : maxc) + 3) & ~3;
-  *cb = m < cap ? m : cap;
-  *two = m > cap;
-}
-
-template <typename T>
-void configure_gram(int) {
-  allow_max_dynamic_smem(gram_kernel<T>);
+int configure_gram(bool f64) {
+  if (f64) return allow_max_dynamic_smem(gram_f64_kernel) >= (int)gram64_smem(GRAM64_CB, 1);
+  int ok = 1;
+#define AP_GT_CFG(NM, NN, DIAG) ok &= allow_max_dynamic_smem(gram_tile_kernel<NM, NN, DIAG>) >= gt_smem<NM, NN, DIAG>()
+  AP_GT_CFG(1, 2, true);
+  AP_GT_CFG(2, 4, true);
+  AP_GT_CFG(3, 6, true);
+  AP_GT_CFG(4, 8, true);
+  AP_GT_CFG(5, 10, true);
+  AP_GT_CFG(6, 12, true);
+  AP_GT_CFG(4, 8, false);
+#undef AP_GT_CFG
+  return ok;
 }
 
 template <typename T>
 void launch_gram(const TileWork* work, const GramRange* ranges, int n_ranges, const int* jt_src,
                  const SourceDev* srcs, const ImageDev* imgs, const T* dbuf, const T* jbuf, const GramPlan& gp,
                  double* vals, int* status, cudaStream_t st, const ForkJoin* fj) {
-  // pass 1: the column-blocking classes write disjoint scratch, so they run
-  // side by side on the auxiliary streams (their launch tails overlap)
+  // pass 1: the launches write disjoint scratch, so they run side by side on
+  // the auxiliary streams (their tails overlap)
   int used = 0;
-  if (fj && n_ranges > 1) cudaEventRecord(fj->fork, st);
+  const bool fork = fj && n_ranges > 1;
+  if (fork) cudaEventRecord(fj->fork, st);
   for (int r = 0; r < n_ranges; ++r) {
     const GramRange& g = ranges[r];
-    if (g.t1 <= g.t0) continue;
+    const int n = g.t1 - g.t0;
+    if (n <= 0) continue;
     cudaStream_t s = st;
-    if (fj && n_ranges > 1) {
+    if (fork) {
       s = fj->aux[used % N_AUX_STREAMS];
       if (used < N_AUX_STREAMS) cudaStreamWaitEvent(s, fj->fork, 0);
       ++used;
     }
     if constexpr (sizeof(T) == 4) {
-      if (g.tc > 0) {
-        launch_gram_tc(g.tc, work, g.t0, g.t1, jt_src, srcs, imgs, reinterpret_cast<const float*>(dbuf),
-                       reinterpret_cast<const float*>(jbuf), gp, status, s);
-        continue;
+      const GramJob* jobs = gp.jobs + g.t0;
+      const float* cbuf = reinterpret_cast<const float*>(jbuf);
+      switch (g.form) {
+        case 1: gt_launch<1, 2, true>(jobs, n, gp, cbuf, status, s); break;
+        case 2: gt_launch<2, 4, true>(jobs, n, gp, cbuf, status, s); break;
+        case 3: gt_launch<3, 6, true>(jobs, n, gp, cbuf, status, s); break;
+        case 4: gt_launch<4, 8, true>(jobs, n, gp, cbuf, status, s); break;
+        case 5: gt_launch<5, 10, true>(jobs, n, gp, cbuf, status, s); break;
+        case 6: gt_launch<6, 12, true>(jobs, n, gp, cbuf, status, s); break;
+        default: gt_launch<4, 8, false>(jobs, n, gp, cbuf, status, s); break;
       }
+    } else {
+      gram_f64_kernel<<<n, TILE_THREADS, gram64_smem(g.form, g.two), s>>>(
+          work, jt_src, srcs, imgs, reinterpret_cast<const double*>(dbuf), reinterpret_cast<const double*>(jbuf), gp.tab0,
+          gp.tab, reinterpret_cast<double*>(gp.scr), g.t0, g.form, g.two);
     }
-    gram_kernel<T><<<g.t1 - g.t0, TILE_THREADS, gram_smem_bytes<T>(g.cb, g.two), s>>>(
-        work, jt_src, srcs, imgs, dbuf, jbuf, gp.tab0, gp.tab, gp.tabs, gp.scr, g.t0, g.cb, g.two, status);
   }
   for (int k = 0; k < used && k < N_AUX_STREAMS; ++k) {
     cudaEventRecord(fj->join[k], fj->aux[k]);
     cudaStreamWaitEvent(st, fj->join[k], 0);
   }
+  using V = typename std::conditional<sizeof(T) == 4, float2, double>::type;
+  const V* scr = reinterpret_cast<const V*>(gp.scr);
   if (gp.n_light > 0) {
     const int blocks = (int)std::min<int64_t>(((int64_t)gp.n_light * 32 + 255) / 256, 8192);
-    gram_reduce_kernel<<<blocks, 256, 0, st>>>(gp.pairs, gp.n_light, gp.pos, gp.scr, vals);
+    gram_reduce_kernel<V><<<blocks, 256, 0, st>>>(gp.pairs, gp.n_light, gp.pos, scr, vals);
   }
-  if (gp.n_heavy_cta > 0)
-    gram_reduce_heavy_kernel<<<gp.n_heavy_cta, 256, 0, st>>>(gp.pairs + gp.n_light, gp.heavy_items, gp.pos, gp.scr,
-                                                             vals);
-  const int n_warp = gp.n_heavy_items - gp.n_heavy_cta;
-  if (n_warp > 0) {
-    // a full wave of 8 CTAs of 8 warps per SM, the warps striding over the list
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int blocks = (int)std::min<int64_t>(((int64_t)n_warp * 32 + 255) / 256, (int64_t)std::max(sms, 1) * 8);
-    gram_reduce_heavy_warp_kernel<<<blocks, 256, 0, st>>>(gp.pairs + gp.n_light, gp.heavy_items + gp.n_heavy_cta,
-                                                          n_warp, gp.pos, gp.scr, vals);
-  }
+  if (gp.n_runs > 0)
+    gram_reduce_run_kernel<V><<<gp.n_runs, 256, 0, st>>>(gp.pairs, gp.runs, gp.pos, scr, gp.part, gp.done, vals);
 }
 
-template void configure_gram<float>(int);
-template void configure_gram<double>(int);
 template void launch_gram<float>(const TileWork*, const GramRange*, int, const int*, const SourceDev*,
                                  const ImageDev*, const float*, const float*, const GramPlan&, double*, int*,
                                  cudaStream_t, const ForkJoin*);
 template void launch_gram<double>(const TileWork*, const GramRange*, int, const int*, const SourceDev*,
                                   const ImageDev*, const double*, const double*, const GramPlan&, double*, int*,
                                   cudaStream_t, const ForkJoin*);
-template void gram_blocking<float>(int, int*, int*);
-template void gram_blocking<double>(int, int*, int*);
 
 }  // namespace ap

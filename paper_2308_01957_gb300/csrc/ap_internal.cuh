@@ -15,7 +15,6 @@ namespace ap {
 constexpr int TILE = 16;
 constexpr int TILE_THREADS = TILE * TILE;
 constexpr int MAX_SLOTS = 8;
-constexpr int GRAM_MAX_COLS = 160;   // Jacobian columns one image tile may hold
 
 // ---------------------------------------------------------------------------
 // device-side descriptors (uploaded once per problem)
@@ -38,6 +37,7 @@ struct ImageDev {
   void* unc;         // H*W:   unconvolved layer U (T)
   void* wr;          // H*W:   w r (T)
   void* wr_trial;    // H*W:   w r at the LM trial point (T)
+  float* sw;         // H*W:   sqrt(w) (float path; written by evaluations that form J^T W J)
   void* adj;         // Hp*Wp: P-correlated w r (T)
   void* psf_flip;    // K*K4:  normalised PSF, flipped, rows padded to K4 (T)
   void* psf_norm;    // K*K4:  normalised PSF, rows padded to K4 (T)
@@ -60,10 +60,23 @@ struct SourceDev {
                      // convolved source's box reaches into the PSF halo)
   int pidx[MAX_SLOTS];
   double pfix[MAX_SLOTS];
-  int64_t d_off;     // element offset of this source's derivative images
+  int64_t d_off;     // element offset of this source's derivative images (-1: none)
   int sup[4];        // Jacobian support: r0, r1, c0, c1 in image pixels
-  int64_t j_off;     // element offset of this source's convolved columns (-1: none)
+  int64_t j_off;     // element offset of this source's convolved columns (float64 path; -1: none)
+  int64_t g_off;     // element offset of this source's column blocks (float path; -1: none)
+  int gt[3];         // column blocks: first tile row, first tile column, tiles per row of the support
+  int nfree;         // free slots
 };
+
+// Column blocks of the float path: a source's free columns, sqrt(w)-scaled,
+// in the image's 16 x 16 tiles -- per tile of its support (row-major), per
+// free slot, the tile's 256 pixels in one kilobyte, zero outside the support.
+// Offset of pixel (i, j) of free slot f:
+__host__ __device__ inline int64_t col_block(const SourceDev& sd, int f, int i, int j) {
+  return sd.g_off +
+         ((int64_t)((i / TILE - sd.gt[0]) * sd.gt[2] + (j / TILE - sd.gt[1])) * sd.nfree + f) * TILE_THREADS +
+         (i % TILE) * TILE + j % TILE;
+}
 
 // Per-evaluation source record, prepared from theta on the device.  A profile
 // (Sersic ... Moffat) works in coordinates scaled by its radius R (Re, sigma,
@@ -110,7 +123,7 @@ struct JcolWork {        // one output tile of one source's Jacobian columns
 
 struct JcolFftWork {     // one FFT block of one free slot of one source's Jacobian columns
   int src;
-  int k;                 // slot
+  int k, f;              // slot, and its rank among the free slots
   int by0, bx0;          // block origin in the source's box coordinates
 };
 
@@ -221,7 +234,7 @@ int configure_live(int Kmax, int is_double);   // shared-memory opt-in of the co
 template <typename T>
 void launch_render_adjoint(int Q, const TileWork* work, int n_work, const int* tile_src,
                            const SourceDev* srcs, const SrcPar<T>* par, const ImageDev* imgs,
-                           double* partial, T* dbuf, cudaStream_t st);
+                           double* partial, T* dbuf, T* cbuf, cudaStream_t st);
 
 // a run of correlation work items sharing one PSF chunk count (K4/4);
 // nc = 0 selects the generic tile code
@@ -235,7 +248,7 @@ int conv_nc_of(int K4, int is_double);
 template <typename T>
 void launch_forward_conv(int tile_variant, const ConvWork* work, const ConvRange* ranges, int n_ranges,
                          const ImageDev* imgs, double* chi2_partial, void* const* model_out, const int* skip,
-                         int trial, int* status, int kmax, cudaStream_t st);
+                         int trial, int store_sw, int* status, int kmax, cudaStream_t st);
 
 // adjoint correlation: adj = P (correlate) w r over the galaxy layer
 template <typename T>
@@ -245,7 +258,7 @@ void launch_adjoint_conv(int tile_variant, const ConvWork* work, const ConvRange
 template <typename T> void configure_conv(int Kmax, int* ok);
 template <typename T>
 void launch_jcol(int variant, const JcolWork* work, const ConvRange* ranges, int n_ranges, const SourceDev* srcs,
-                 const ImageDev* imgs, const T* dbuf, T* jbuf, int kmax, cudaStream_t st);
+                 const ImageDev* imgs, const T* dbuf, T* jbuf, int kmax, cudaStream_t st);   // jbuf: columns (float: column blocks)
 // FFT mode of the Jacobian-column convolution (float only; see ap_fft.cu)
 constexpr int FFT_MAX_K64 = 33, FFT_MAX_K128 = 97;   // largest PSF per FFT block size (B >= 32)
 int configure_fft();
@@ -254,9 +267,6 @@ void launch_psf_spectrum(int N, const float* psf_norm, int K, int K4, const floa
                          cudaStream_t st);
 void launch_jcol_fft(int N, const JcolFftWork* work, int n, const SourceDev* srcs, const ImageDev* imgs,
                      const float* dbuf, float* jbuf, const float2* tw, cudaStream_t st);
-template <typename T> void configure_gram(int unused);
-template <typename T> void gram_blocking(int maxc, int* cb, int* two);
-int gram_max_cols(int is_double);
 int conv_tile_w(int variant);
 int conv_tile_h(int variant);
 int conv_threads(int variant);
@@ -278,48 +288,47 @@ struct GramPair {
   int excl;       // 1: no other pair adds to its CSR entries (plain stores)
 };
 
-// A pair meeting more than GRAM_HEAVY_TILES tiles keeps its scratch entry
-// by entry (the tiles of one entry contiguous); each entry is summed by one
-// warp, or by a whole CTA when it spans more than GRAM_CTA_TILES tiles (a
-// source and the sky, the sky and itself).  The other pairs keep it tile by
-// tile and are summed by one warp per pair.
-constexpr int GRAM_HEAVY_TILES = 64;
-constexpr int GRAM_CTA_TILES = 2048;
-
-struct GramRange {     // tiles [t0, t1) of the tile list share one column blocking
-  int t0, t1, cb, two;
-  int tc;              // float path: tcgen05 kernel form (gram_tc_kind: 1, 2, 3), 0 = warp MMA
+// Pass 2 sums a pair of up to GRAM_LIGHT_VALUES values with one warp and cuts
+// the others into runs of some GRAM_RUN_VALUES values, a CTA each.
+constexpr int GRAM_LIGHT_VALUES = 2048;
+constexpr int GRAM_RUN_VALUES = 8192;
+struct GramRun {
+  int pair;
+  int k0, k1;          // tiles of the pair
+  int first, run, n_runs;   // index of the pair's first run, this one's rank, their number
 };
 
-// One free Jacobian column of a tile, as the tensor-core tile Gram reads it
-// (planned on the host): the column image at element offset `off` of the
-// convolved-column buffer (info bit 30 set) or of the derivative buffer, its
-// row pitch bw, the offset off0 of the tile's pixel (0, 0) in it (may lie
-// outside the image), its box in tile coordinates clamped to 0..16 (rows
-// [b0, b1), columns [b2, b3), a byte each) and
-// info = (local source << 8) | (free slot << 4) | free slots of the source.
-struct GramCol {
-  int64_t off;
-  int off0;
-  int bw;
-  uint32_t bounds;
-  int info;
+struct GramRange {     // float path: jobs [t0, t1) of one kernel form; float64 path: tiles
+  int t0, t1;          //   [t0, t1) sharing one column blocking (form = columns of a block)
+  int form, two;
 };
-constexpr int GRAM_COL_CONV = 1 << 30;
+
+// float path: one source of a tile's list as the tile Gram reads it
+struct GramEnt {
+  int64_t off;         // its column blocks of this tile
+  int nf, col0;        // free columns, and the first one's index among the tile's columns
+};
+// float path: columns [ca0, ca0 + na) against [cb0, cb0 + nb) of a tile
+struct GramJob {
+  int64_t tab0;        // the tile's pair table
+  int e0, L;           // its source list
+  int ca0, na, cb0, nb;
+};
+constexpr int GRAM_FORMS = 7;
 
 struct GramPlan {
   const int64_t* tab0;   // per tile: first entry of its pair table
   const int64_t* tab;    // per tile, per local pair (a <= b): scratch offset of its block
-  const int* tabs;       //   and the stride between the block's entries (1, or the pair's tile count)
-  double* scr;           // per-tile pair blocks
-  const GramPair* pairs; // light pairs first, then the heavy ones
+  void* scr;             // per-tile pair blocks (float path: float2 hi + lo; float64 path: double)
+  const GramPair* pairs; // light pairs first, then the others
   const int64_t* pos;    // CSR positions of the pair blocks' entries
-  int n_light, n_heavy;
-  const int* heavy_items; // (heavy pair << 6) | entry, for every stored entry of the heavy pairs:
-  int n_heavy_items;      //   first the n_heavy_cta entries summed by a CTA each, then those summed by a warp
-  int n_heavy_cta;
-  const int64_t* col_ptr; // float path: per tile, its first column in cols (with a closing entry)
-  const GramCol* cols;    //   the tiles' free columns in (source, slot) order
+  int n_light;
+  const GramRun* runs;   // runs of the other pairs
+  int n_runs;
+  double* part;          // 64 partial sums per run
+  int* done;             // finished runs per pair (at its first run's index); zero between calls
+  const GramJob* jobs;   // float path
+  const GramEnt* ents;   // float path: parallel to the tiles' source lists
 };
 
 // independent launches forked from a stream onto auxiliary streams and
@@ -331,17 +340,12 @@ struct ForkJoin {
   cudaEvent_t join[N_AUX_STREAMS];
 };
 
-// tcgen05 tile Grams (float path, tiles of up to gram_tc_max_cols() columns;
-// see ap_gram_tc.cu)
-int gram_tc_max_cols();
-constexpr int GRAM_TC_MIN_DEFAULT = 33;   // before the planner has timed the two kernels
-// kernel form of a tile of `cols` columns: 1 (up to 64), 2 (up to 128), 3 (up to 256)
-int gram_tc_kind(int cols);
-void configure_gram_tc();
-void launch_gram_tc(int kind, const TileWork* work, int t0, int t1, const int* jt_src, const SourceDev* srcs,
-                    const ImageDev* imgs, const float* dbuf, const float* jbuf, const GramPlan& gp, int* status,
-                    cudaStream_t st);
-
+int configure_gram(bool f64);
+void gram_plan_jobs(const std::vector<TileWork>& tiles, const std::vector<int64_t>& tab0,
+                    const std::vector<int>& tile_ncol, std::vector<GramJob>& jobs, std::vector<GramRange>& ranges);
+void gram64_blocking(int maxc, int* cb, int* two);
+// dbuf / jbuf: derivative images and convolved columns (float64 path); the
+// float path reads the column blocks in jbuf alone
 template <typename T>
 void launch_gram(const TileWork* work, const GramRange* ranges, int n_ranges, const int* jt_src,
                  const SourceDev* srcs, const ImageDev* imgs, const T* dbuf, const T* jbuf, const GramPlan& gp,

@@ -735,11 +735,25 @@ __device__ __forceinline__ T warp_sum_slots(const T (&v)[MAX_SLOTS], int lane) {
 // every warp to the slowest one of each).
 constexpr int ADJ_RUN = 16;
 
+// an unconvolved source's derivatives are its Jacobian columns: sqrt(w)-scaled
+// into its column blocks (float path; the tile of the unconvolved layer is the
+// block's)
+__device__ __forceinline__ void store_columns(float* cbuf, const SourceDev& sd, int i, int j, float sw,
+                                              const float (&D)[MAX_SLOTS]) {
+  float* dst = cbuf + col_block(sd, 0, i, j);
+#pragma unroll
+  for (int k = 0; k < MAX_SLOTS; ++k)
+    if (k < sd.nslot && sd.pidx[k] >= 0) {
+      *dst = D[k] * sw;
+      dst += TILE_THREADS;
+    }
+}
+
 template <typename T, int Q>
 __global__ void __launch_bounds__(RENDER_THREADS) render_adjoint_kernel(
     const TileWork* __restrict__ work, const int* __restrict__ tile_src, const SourceDev* __restrict__ srcs,
     const SrcPar<T>* __restrict__ par, const ImageDev* __restrict__ imgs, double* __restrict__ partial,
-    T* __restrict__ dbuf) {
+    T* __restrict__ dbuf, T* __restrict__ cbuf) {
   constexpr int NW = RENDER_THREADS / 32;
   __shared__ T red[ADJ_RUN][NW][MAX_SLOTS];
   const TileWork w = work[blockIdx.x];
@@ -755,6 +769,11 @@ __global__ void __launch_bounds__(RENDER_THREADS) render_adjoint_kernel(
   const T* a = (const T*)(w.plane == 0 ? im.adj : im.wr);
   const T adj0 = ok0 ? a[(size_t)(i0 + h) * cols + (j + h)] : (T)0;
   const T adj1 = ok1 ? a[(size_t)(i1 + h) * cols + (j + h)] : (T)0;
+  float sw0 = 0.f, sw1 = 0.f;
+  if (sizeof(T) == 4 && cbuf != nullptr && w.plane == 1) {
+    if (ok0) sw0 = im.sw[(size_t)i0 * im.W + j];
+    if (ok1) sw1 = im.sw[(size_t)i1 * im.W + j];
+  }
   for (int e0 = w.e0; e0 < w.e1; e0 += ADJ_RUN) {
     const int ne = min(ADJ_RUN, w.e1 - e0);
     for (int k0 = 0; k0 < ne; ++k0) {
@@ -789,6 +808,12 @@ __global__ void __launch_bounds__(RENDER_THREADS) render_adjoint_kernel(
           if (in0) store_derivs(dbuf, sd, i0, j, D0);
           if (in1) store_derivs(dbuf, sd, i1, j, D1);
         }
+        if constexpr (sizeof(T) == 4) {
+          if (cbuf != nullptr && w.plane == 1 && sd.g_off >= 0) {
+            if (in0) store_columns(cbuf, sd, i0, j, sw0, D0);
+            if (in1) store_columns(cbuf, sd, i1, j, sw1, D1);
+          }
+        }
       }
       __syncwarp();
       // the warp's sum over its 64 pixels in T; the per-tile partial joins
@@ -809,13 +834,14 @@ __global__ void __launch_bounds__(RENDER_THREADS) render_adjoint_kernel(
 
 template <typename T>
 void launch_render_adjoint(int Q, const TileWork* work, int n_work, const int* tile_src, const SourceDev* srcs,
-                           const SrcPar<T>* par, const ImageDev* imgs, double* partial, T* dbuf, cudaStream_t st) {
+                           const SrcPar<T>* par, const ImageDev* imgs, double* partial, T* dbuf, T* cbuf,
+                           cudaStream_t st) {
   if (n_work <= 0) return;
   switch (Q) {
-    case 1: render_adjoint_kernel<T, 1><<<n_work, RENDER_THREADS, 0, st>>>(work, tile_src, srcs, par, imgs, partial, dbuf); break;
-    case 3: render_adjoint_kernel<T, 3><<<n_work, RENDER_THREADS, 0, st>>>(work, tile_src, srcs, par, imgs, partial, dbuf); break;
-    case 5: render_adjoint_kernel<T, 5><<<n_work, RENDER_THREADS, 0, st>>>(work, tile_src, srcs, par, imgs, partial, dbuf); break;
-    default: render_adjoint_kernel<T, 7><<<n_work, RENDER_THREADS, 0, st>>>(work, tile_src, srcs, par, imgs, partial, dbuf); break;
+    case 1: render_adjoint_kernel<T, 1><<<n_work, RENDER_THREADS, 0, st>>>(work, tile_src, srcs, par, imgs, partial, dbuf, cbuf); break;
+    case 3: render_adjoint_kernel<T, 3><<<n_work, RENDER_THREADS, 0, st>>>(work, tile_src, srcs, par, imgs, partial, dbuf, cbuf); break;
+    case 5: render_adjoint_kernel<T, 5><<<n_work, RENDER_THREADS, 0, st>>>(work, tile_src, srcs, par, imgs, partial, dbuf, cbuf); break;
+    default: render_adjoint_kernel<T, 7><<<n_work, RENDER_THREADS, 0, st>>>(work, tile_src, srcs, par, imgs, partial, dbuf, cbuf); break;
   }
 }
 
@@ -1537,7 +1563,7 @@ template void launch_prepare<double>(const SourceDev*, const ImageDev*, int, con
                                      const int*, int*, cudaStream_t);
 template void launch_render<float>(int, const TileWork*, int, const int*, const SourceDev*, const SrcPar<float>*, const ImageDev*, const int*, cudaStream_t);
 template void launch_render<double>(int, const TileWork*, int, const int*, const SourceDev*, const SrcPar<double>*, const ImageDev*, const int*, cudaStream_t);
-template void launch_render_adjoint<float>(int, const TileWork*, int, const int*, const SourceDev*, const SrcPar<float>*, const ImageDev*, double*, float*, cudaStream_t);
-template void launch_render_adjoint<double>(int, const TileWork*, int, const int*, const SourceDev*, const SrcPar<double>*, const ImageDev*, double*, double*, cudaStream_t);
+template void launch_render_adjoint<float>(int, const TileWork*, int, const int*, const SourceDev*, const SrcPar<float>*, const ImageDev*, double*, float*, float*, cudaStream_t);
+template void launch_render_adjoint<double>(int, const TileWork*, int, const int*, const SourceDev*, const SrcPar<double>*, const ImageDev*, double*, double*, double*, cudaStream_t);
 
 }  // namespace ap
