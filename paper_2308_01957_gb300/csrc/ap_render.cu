@@ -471,7 +471,7 @@ __device__ __forceinline__ T pixel_value(int type, const SrcPar<T>& P, int i, in
         const T x = xb + P.m00 * ha, y = yb + P.m10 * ha;
         const T u = fma(x, x, fma(y, y, P.k1));
         const T t = p_exp2(P.k0 * p_log2(u));                 // (R/Re)^(1/n)
-        accb += gl_hw<T>(Q, a) * p_exp2(fma(-P.k2, t, P.k2));  // exp(-b (t - 1))
+        accb += gl_hw<T>(Q, a) * p_exp2(fma(-P.k2, t, P.k2));
       }
     } else if (type == AP_GAUSSIAN) {
 #pragma unroll
@@ -626,7 +626,7 @@ __device__ __forceinline__ void pixel_derivs(int type, const SrcPar<T>& P, int i
         const T lt = P.k0 * p_log2(u);            // log2 t
         const T t = p_exp2(lt);                   // (R/Re)^(1/n)
         const T v = (T)1 - t;
-        const T we = (wb * gl_hw<T>(Q, a)) * p_exp2(P.k2 * v);   // w exp(-b (t - 1))
+        const T we = (wb * gl_hw<T>(Q, a)) * p_exp2(fma(-P.k2, t, P.k2));   // w exp(-b (t - 1))
         const T wt = we * t;
         const T g = wt * p_rcp(u);
         S1 += we;
