@@ -134,7 +134,6 @@ struct ap_ctx {
   double* d_chi2_trial = nullptr;
   double* d_chi2_state = nullptr;
   double* d_lambda = nullptr;
-  int* d_accepted = nullptr;
   int* d_cg_iters = nullptr;
   double* d_log = nullptr;
   int* d_log_iter = nullptr;
@@ -300,8 +299,9 @@ void param_bounds(const std::vector<SourceDev>& srcs, int n_params, std::vector<
 // and everything after it run for every group.  trial: the forward state goes
 // to the trial buffers (d_par_trial, wr_trial), leaving the current point's.
 template <typename T>
-int do_eval(ap_ctx* c, const double* theta, double* chi2_out, double* grad_out, void* const* model_ptrs_dev,
-            bool want_D, const int* skip, bool trial, cudaStream_t st) {
+int do_eval(ap_ctx* c, const double* theta, double* chi2_out, double* grad_out, double* jtwr_out,
+            void* const* model_ptrs_dev, const int* skip, bool trial, cudaStream_t st) {
+  const bool want_D = jtwr_out != nullptr;
   SrcPar<T>* par = (SrcPar<T>*)(trial ? c->d_par_trial : c->d_par);
   c->launches_last_eval = (c->n_src > 0) + (c->n_rwork > 0) + (c->n_fwork > 0) + (chi2_out && c->n_groups > 0) +
                           (grad_out ? (c->n_awork > 0) + (c->n_rwork > 0) + (c->n_params > 0) : 0);
@@ -348,16 +348,17 @@ int do_eval(ap_ctx* c, const double* theta, double* chi2_out, double* grad_out, 
     }
     {
       Bracket b(c, st, "grad_gather");
-      launch_sum_contrib(c->d_grad_partial, c->d_gc_ptr, c->d_gc_idx, c->n_params, grad_out, -2.0, st);
+      launch_sum_contrib(c->d_grad_partial, c->d_gc_ptr, c->d_gc_idx, c->n_params, grad_out, -2.0, jtwr_out, st);
     }
   }
   return AP_OK;
 }
 
-int eval_any(ap_ctx* c, const double* theta, double* chi2_out, double* grad_out, void* const* model_ptrs_dev,
-             bool want_D, cudaStream_t st, const int* skip = nullptr, bool trial = false) {
-  return c->f64 ? do_eval<double>(c, theta, chi2_out, grad_out, model_ptrs_dev, want_D, skip, trial, st)
-                : do_eval<float>(c, theta, chi2_out, grad_out, model_ptrs_dev, want_D, skip, trial, st);
+// jtwr_out (nullable, with grad_out): J^T W r, and the derivative images are kept
+int eval_any(ap_ctx* c, const double* theta, double* chi2_out, double* grad_out, double* jtwr_out,
+             void* const* model_ptrs_dev, cudaStream_t st, const int* skip = nullptr, bool trial = false) {
+  return c->f64 ? do_eval<double>(c, theta, chi2_out, grad_out, jtwr_out, model_ptrs_dev, skip, trial, st)
+                : do_eval<float>(c, theta, chi2_out, grad_out, jtwr_out, model_ptrs_dev, skip, trial, st);
 }
 
 void launch_jcol_fft_all(ap_ctx* c, cudaStream_t st) {
@@ -380,12 +381,8 @@ void launch_jcol_fft_all(ap_ctx* c, cudaStream_t st) {
 }
 
 int normal_eq_any(ap_ctx* c, const double* theta, double* jtwr_out, cudaStream_t st, const int* skip = nullptr) {
-  int rc = eval_any(c, theta, c->d_chi2, c->d_grad, nullptr, true, st, skip);
+  int rc = eval_any(c, theta, c->d_chi2, c->d_grad, jtwr_out, nullptr, st, skip);
   if (rc) return rc;
-  {
-    Bracket b(c, st, "jtwr_scale");
-    launch_scale(c->d_grad, jtwr_out, -0.5, c->n_params, st);
-  }
   cudaMemsetAsync(c->d_vals, 0, (size_t)std::max<int64_t>(c->nnz, 1) * sizeof(double), st);
   {
     Bracket b(c, st, "jacobian_columns");
@@ -443,14 +440,12 @@ int lm_iteration(ap_ctx* c, cudaStream_t st) {
     Bracket b(c, st, "lm_trial");
     launch_trial(c->d_theta, c->d_delta, c->d_lo, c->d_hi, c->d_trial, c->n_params, st);
   }
-  rc = eval_any(c, c->d_trial, c->d_chi2_trial, nullptr, nullptr, false, st, nullptr, true);
+  rc = eval_any(c, c->d_trial, c->d_chi2_trial, nullptr, nullptr, nullptr, st, nullptr, true);
   if (rc) return rc;
   {
     Bracket b(c, st, "lm_accept");
-    launch_accept_groups(c->d_chi2, c->d_chi2_trial, c->d_lambda, c->d_chi2_state, c->d_log, c->d_accepted,
-                         c->d_fwd_valid, c->n_groups, st);
-    launch_accept_params(c->d_param_group, c->n_params, c->d_accepted, c->d_theta, c->d_trial, st);
-    launch_accept_state(c->d_state_chunks, c->n_state_chunks, c->d_accepted, st);
+    launch_accept(c->d_chi2, c->d_chi2_trial, c->d_lambda, c->d_chi2_state, c->d_log, c->d_fwd_valid, c->n_groups,
+                  c->d_param_group, c->n_params, c->d_theta, c->d_trial, c->d_state_chunks, c->n_state_chunks, st);
   }
   return AP_OK;
 }
@@ -671,7 +666,7 @@ int lm_run(ap_ctx* c, double* theta, double* lambda, double* chi2, int n_iter, d
     if (n_iter > 0) {
       CUDA_TRY(c, cudaMemcpyAsync(chi2, c->d_chi2_state, G * sizeof(double), cudaMemcpyDeviceToDevice, st));
     } else {
-      int rc = eval_any(c, c->d_theta, chi2, nullptr, nullptr, false, st);
+      int rc = eval_any(c, c->d_theta, chi2, nullptr, nullptr, nullptr, st);
       if (rc) return rc;
       if ((rc = drop_lm_reuse(c, st))) return rc;
     }
@@ -1650,8 +1645,6 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
   double** gv[] = {&c->d_chi2, &c->d_chi2_trial, &c->d_chi2_state, &c->d_lambda};
   for (double** v : gv)
     if ((rc = dev_alloc(c, (void**)v, G * sizeof(double)))) return rc;
-  if ((rc = dev_alloc(c, (void**)&c->d_accepted, G * sizeof(int)))) return rc;
-  CUDA_TRY(c, cudaMemset(c->d_accepted, 0, G * sizeof(int)));
   if ((rc = dev_alloc(c, (void**)&c->d_fwd_valid, G * sizeof(int)))) return rc;
   CUDA_TRY(c, cudaMemset(c->d_fwd_valid, 0, G * sizeof(int)));
   if ((rc = dev_alloc(c, (void**)&c->d_cg_iters, G * sizeof(int)))) return rc;
@@ -1973,7 +1966,7 @@ int ap_render(ap_ctx* c, const double* theta, void* const* model_dev, void* stre
   cudaSetDevice(c->opt.device);
   cudaStream_t st = (cudaStream_t)stream;
   launch_store_ptrs(model_dev, c->n_img, c->d_model_ptrs, st);
-  int rc = eval_any(c, theta, nullptr, nullptr, c->d_model_ptrs, false, st);
+  int rc = eval_any(c, theta, nullptr, nullptr, nullptr, c->d_model_ptrs, st);
   if (rc) return rc;
   if ((rc = drop_lm_reuse(c, st))) return rc;
   CUDA_TRY(c, cudaGetLastError());
@@ -1984,7 +1977,7 @@ int ap_eval(ap_ctx* c, const double* theta, double* chi2, double* grad, void* st
   if (!c || !theta || !chi2) return AP_ERR_ARG;
   if (!c->have_problem) return fail(c, AP_ERR_STATE, "no problem set");
   cudaStream_t st = (cudaStream_t)stream;
-  int rc = eval_any(c, theta, chi2, grad, nullptr, false, st);
+  int rc = eval_any(c, theta, chi2, grad, nullptr, nullptr, st);
   if (rc) return rc;
   if ((rc = drop_lm_reuse(c, st))) return rc;
   CUDA_TRY(c, cudaGetLastError());

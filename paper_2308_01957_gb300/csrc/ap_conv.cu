@@ -487,54 +487,68 @@ void launch_jcol(int v, const JcolWork* work, const ConvRange* ranges, int n_ran
 }
 
 // ---------------------------------------------------------------------------
-// deterministic float64 gathers: one warp per output, lanes stride over the
-// output's list in a fixed order, then a fixed shuffle tree
+// deterministic float64 gathers: one CTA per output (its list may be long: a
+// group's correlation tiles, a sky parameter's render tiles), the threads stride
+// over the list in a fixed order, then a fixed tree
 // ---------------------------------------------------------------------------
-__global__ void sum_groups_kernel(const double* __restrict__ partial, const int* __restrict__ ptr,
-                                  const int* __restrict__ idx, int n_out, double* __restrict__ out, double scale,
-                                  const int* __restrict__ skip, const double* __restrict__ keep) {
-  const int g = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  const int lane = threadIdx.x & 31;
-  if (g >= n_out) return;
-  if (skip && skip[g]) {   // the group's forward did not run: its value is kept
-    if (lane == 0) out[g] = keep[g];
-    return;
-  }
-  double s = 0.0;
-  for (int k = ptr[g] + lane; k < ptr[g + 1]; k += 32) s += partial[idx[k]];
+template <int NT, class I>
+__device__ __forceinline__ double gather_sum(const double* __restrict__ partial, const I* __restrict__ idx, I k0, I k1,
+                                             double* red) {
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  for (I k = k0 + threadIdx.x; k < k1; k += 4 * NT) {   // four independent gathers in flight
+    I at[4];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) out[g] = scale * s;
+    for (int u = 0; u < 4; ++u) at[u] = k + u * NT < k1 ? idx[k + u * NT] : (I)-1;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s[u] += at[u] >= 0 ? partial[at[u]] : 0.0;
+  }
+  double v = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < NT / 32; ++w) v += red[w];
+  return v;   // thread 0
 }
 
-// one 128-thread block per output: the list may be long (a sky parameter has
-// one entry per tile it covers)
+constexpr int SUM_GROUP_THREADS = 256;
+__global__ void __launch_bounds__(SUM_GROUP_THREADS) sum_groups_kernel(
+    const double* __restrict__ partial, const int* __restrict__ ptr, const int* __restrict__ idx,
+    double* __restrict__ out, double scale, const int* __restrict__ skip, const double* __restrict__ keep) {
+  __shared__ double red[SUM_GROUP_THREADS / 32];
+  const int g = blockIdx.x;
+  if (skip && skip[g]) {   // the group's forward did not run: its value is kept
+    if (threadIdx.x == 0) out[g] = keep[g];
+    return;
+  }
+  const double s = gather_sum<SUM_GROUP_THREADS, int>(partial, idx, ptr[g], ptr[g + 1], red);
+  if (threadIdx.x == 0) out[g] = scale * s;
+}
+
 __global__ void __launch_bounds__(128) sum_contrib_kernel(const double* __restrict__ partial,
                                                           const int64_t* __restrict__ ptr,
-                                                          const int64_t* __restrict__ idx, int n_out,
-                                                          double* __restrict__ out, double scale) {
+                                                          const int64_t* __restrict__ idx, double* __restrict__ out,
+                                                          double scale, double* __restrict__ half) {
   __shared__ double red[4];
   const int g = blockIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double s = 0.0;
-  for (int64_t k = ptr[g] + threadIdx.x; k < ptr[g + 1]; k += 128) s += partial[idx[k]];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) red[warp] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) out[g] = scale * (((red[0] + red[1]) + red[2]) + red[3]);
+  const double s = gather_sum<128, int64_t>(partial, idx, ptr[g], ptr[g + 1], red);
+  if (threadIdx.x == 0) {
+    out[g] = scale * s;
+    if (half) half[g] = -0.5 * (scale * s);
+  }
 }
 
 void launch_sum_groups(const double* partial, const int* ptr, const int* idx, int n_out, double* out, double scale,
                        const int* skip, const double* keep, cudaStream_t st) {
-  if (n_out <= 0) return;
-  sum_groups_kernel<<<(n_out + 7) / 8, 256, 0, st>>>(partial, ptr, idx, n_out, out, scale, skip, keep);
+  if (n_out > 0)
+    sum_groups_kernel<<<n_out, SUM_GROUP_THREADS, 0, st>>>(partial, ptr, idx, out, scale, skip, keep);
 }
 
 void launch_sum_contrib(const double* partial, const int64_t* ptr, const int64_t* idx, int n_out, double* out,
-                        double scale, cudaStream_t st) {
-  if (n_out <= 0) return;
-  sum_contrib_kernel<<<n_out, 128, 0, st>>>(partial, ptr, idx, n_out, out, scale);
+                        double scale, double* half, cudaStream_t st) {
+  if (n_out > 0) sum_contrib_kernel<<<n_out, 128, 0, st>>>(partial, ptr, idx, out, scale, half);
 }
 
 template void configure_conv<float>(int, int*);

@@ -274,8 +274,9 @@ constexpr int N_CONV_VARIANTS = 7;
 
 void launch_sum_groups(const double* partial, const int* ptr, const int* idx, int n_out, double* out,
                        double scale, const int* skip, const double* keep, cudaStream_t st);
+// out = scale * sum; half (nullable): -sum * scale / 2, the J^T W r of a gradient
 void launch_sum_contrib(const double* partial, const int64_t* ptr, const int64_t* idx, int n_out, double* out,
-                        double scale, cudaStream_t st);
+                        double scale, double* half, cudaStream_t st);
 
 // J^T W J in two passes (see ap_gram.cu).  A source pair is two sources
 // (A <= B) reaching a common image tile; its block holds the m_A x m_B
@@ -449,15 +450,6 @@ int launch_pcg_dist(const GroupDev* groups_host, int n_groups, const SolvePlan& 
 
 void launch_trial(const double* theta, const double* delta, const double* lo, const double* hi,
                   double* trial, int n, cudaStream_t st);
-void launch_accept(const int* param_group, int n_params, const double* chi2_now, const double* chi2_trial,
-                   double* theta, const double* trial, double* lambda, double* chi2_state, double* log,
-                   int n_groups, cudaStream_t st);
-void launch_accept_params(const int* param_group, int n_params, const int* accepted, double* theta,
-                          const double* trial, cudaStream_t st);
-void launch_accept_groups(const double* chi2_now, const double* chi2_trial, double* lambda,
-                          double* chi2_state, double* log, int* accepted, int* fwd_valid, int n_groups,
-                          cudaStream_t st);
-
 // A run of 32-bit words of the trial point's forward state (source records,
 // w r) and where it goes when the group accepts: the copy makes them the
 // current point's.
@@ -467,9 +459,10 @@ struct StateChunk {
   int n_words;
   int group;
 };
-constexpr int STATE_CHUNK_WORDS = 16384;
-void launch_accept_state(const StateChunk* chunks, int n_chunks, const int* accepted, cudaStream_t st);
-void launch_scale(const double* in, double* out, double s, int n, cudaStream_t st);
+constexpr int STATE_CHUNK_WORDS = 4096;
+void launch_accept(const double* chi2_now, const double* chi2_trial, double* lambda, double* chi2_state, double* log,
+                   int* fwd_valid, int n_groups, const int* param_group, int n_params, double* theta,
+                   const double* trial, const StateChunk* chunks, int n_chunks, cudaStream_t st);
 // dst_dev[0..n) = src_host[0..n), stream-ordered, the values passed in kernel
 // arguments (runs of PTR_RUN pointers per launch)
 constexpr int PTR_RUN = 256;

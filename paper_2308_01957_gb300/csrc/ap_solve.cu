@@ -10,13 +10,15 @@
 // AP_ERR_NOT_SPD and delta_g = 0.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "ap_internal.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace ap {
 
-constexpr int CHOL_THREADS = 256;
+constexpr int CHOL_THREADS = 128;
 constexpr int PCG_THREADS = 1024;
 constexpr int LM_RETRIES = 8;
 constexpr double DIAG_FLOOR = 1e-12;
@@ -28,7 +30,7 @@ constexpr double PCG_RTOL = 1e-11;
 // Block reductions: warp shuffles, then warp 0 combines the warp partials
 // with a fixed shuffle tree and broadcasts through shared memory (one warp
 // does the float64 adds, not every thread).  red[] holds 33 doubles.
-__device__ double block_sum(double v, double* red) {
+__device__ __forceinline__ double block_sum(double v, double* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = (blockDim.x + 31) >> 5;
 #pragma unroll
@@ -46,7 +48,7 @@ __device__ double block_sum(double v, double* red) {
   return red[32];
 }
 
-__device__ double block_max(double v, double* red) {
+__device__ __forceinline__ double block_max(double v, double* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = (blockDim.x + 31) >> 5;
 #pragma unroll
@@ -65,98 +67,113 @@ __device__ double block_max(double v, double* red) {
 }
 
 // ---------------------------------------------------------------------------
-// dense Cholesky, one CTA per small group; matrix in shared memory
+// dense factorisation of a small group (up to 64 parameters), one CTA each; the
+// matrix in shared memory.
+//
+// Cholesky in the form L diag(d) L^T (the same pivots, no square roots), right
+// looking, one barrier per column: a thread owns a row (two threads share its
+// columns) and updates it with the column's unscaled entries; the scaled ones go to
+// the upper triangle; the thread that completes the next pivot also takes its
+// reciprocal (in every thread, the divisions would take as long as the updates).
+// The right-hand side rides along as row n, which makes the forward substitution
+// part of the factorisation; one warp does the back substitution by columns.
+// Bound by the float64 pipe (a warp's FMA holds it for some 17 clocks, n^3 / 170
+// of them) and the column's latency chain.  64 groups of up to 57 parameters
+// 240 -> 90 us, one of 8 parameters 21 -> 9 us (divisions per element, an index
+// division per update and a one-thread substitution took the time).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(CHOL_THREADS) chol_kernel(const GroupDev* __restrict__ groups, int n_groups,
-                                                            const int* __restrict__ gparams,
-                                                            const int* __restrict__ plocal,
-                                                            const int64_t* __restrict__ row_ptr,
-                                                            const int32_t* __restrict__ col_idx,
-                                                            const double* __restrict__ vals,
-                                                            const double* __restrict__ jtwr, double* lambda,
-                                                            double* delta, int max_n, int* status) {
+__host__ __device__ inline int chol_pitch(int n) { return n | 1; }   // odd: rows on different banks
+
+__global__ void __launch_bounds__(CHOL_THREADS) chol_kernel(
+    const GroupDev* __restrict__ groups, const int* __restrict__ gparams, const int64_t* __restrict__ row_ptr,
+    const int32_t* __restrict__ lcol, const int64_t* __restrict__ dpos, const double* __restrict__ vals,
+    const double* __restrict__ jtwr, double* lambda, double* delta, int max_n, int* status) {
   extern __shared__ double sm[];
   __shared__ double red[33];
-  __shared__ int fail;
   const int g = blockIdx.x;
   const GroupDev G = groups[g];
   if (G.dense != 1) return;
-  const int n = G.n;
+  const int n = G.n, P = chol_pitch(n);
   const int* gp = gparams + G.p0;
-  double* A = sm;               // n x n damped copy
-  double* A0 = A + max_n * max_n;   // n x n original
-  double* D = A0 + max_n * max_n;   // n
-  double* y = D + max_n;            // n
-  const int tid = threadIdx.x;
-  for (int idx = tid; idx < n * n; idx += blockDim.x) A0[idx] = 0.0;
-  __syncthreads();
-  for (int r = tid; r < n; r += blockDim.x) {
-    const int pr = gp[r];
-    for (int64_t e = row_ptr[pr]; e < row_ptr[pr + 1]; ++e) {
-      const int lc = plocal[col_idx[e]];
-      if (lc >= 0 && lc < n) A0[r * n + lc] = vals[e];
-    }
+  double* A = sm;                                        // rows 0..n - 1, and the right-hand side as row n
+  double* D = A + (max_n + 1) * chol_pitch(max_n);       // damping diagonal
+  double* z = D + max_n;                                 // D^-1 L^-1 b
+  double* inv = z + max_n;                               // reciprocal pivots, 0 where the pivot fails
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // hardware seed (20 bits) and two Newton steps, r <- r + r (1 - d r)
+  auto reciprocal = [](double d) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    r = fma(r, fma(-d, r, 1.0), r);
+    r = fma(r, fma(-d, r, 1.0), r);
+    return d > 0.0 && isfinite(d) && isfinite(r) ? r : 0.0;
+  };
+  double d0 = 0.0;
+  if (tid < n) {
+    const int64_t e = dpos[gp[tid]];
+    d0 = e >= 0 ? vals[e] : 0.0;
   }
-  __syncthreads();
-  double dmax = 0.0;
-  for (int r = tid; r < n; r += blockDim.x) dmax = fmax(dmax, A0[r * n + r]);
-  dmax = block_max(dmax, red);
-  const double floor_v = dmax > 0.0 ? DIAG_FLOOR * dmax : 1.0;
-  for (int r = tid; r < n; r += blockDim.x) D[r] = fmax(A0[r * n + r], floor_v);
+  const double dmax = block_max(fmax(d0, 0.0), red);
+  if (tid < n) D[tid] = fmax(d0, dmax > 0.0 ? DIAG_FLOOR * dmax : 1.0);
   double lam = lambda[g];
   bool ok = false;
-  for (int attempt = 0; attempt <= LM_RETRIES; ++attempt) {
+  for (int attempt = 0; attempt <= LM_RETRIES && !ok; ++attempt) {
     __syncthreads();
-    for (int idx = tid; idx < n * n; idx += blockDim.x) {
-      const int r = idx / n, c = idx - r * n;
-      A[idx] = A0[idx] + (r == c ? lam * D[r] : 0.0);
+    for (int idx = tid; idx < n * P; idx += CHOL_THREADS) A[idx] = 0.0;
+    if (tid < n) A[n * P + tid] = jtwr[gp[tid]];
+    __syncthreads();
+    for (int r = warp; r < n; r += CHOL_THREADS / 32) {
+      const int pr = gp[r];
+      for (int64_t e = row_ptr[pr] + lane; e < row_ptr[pr + 1]; e += 32) {
+        const int c = lcol[e];
+        if (c >= 0 && c <= r) A[r * P + c] = vals[e];
+      }
     }
-    if (tid == 0) fail = 0;
     __syncthreads();
-    // right-looking column Cholesky, lower triangle
+    if (tid < n) A[tid * P + tid] += lam * D[tid];
+    if (tid == 0 && n > 0) inv[0] = reciprocal(A[0]);
+    __syncthreads();
+    ok = true;
     for (int k = 0; k < n; ++k) {
-      if (tid == 0) {
-        const double d = A[k * n + k];
-        if (!(d > 0.0) || !isfinite(d)) fail = 1;
-        else A[k * n + k] = sqrt(d);
+      const double iv = inv[k];
+      if (iv == 0.0) {   // the same for every thread
+        ok = false;
+        break;
       }
-      __syncthreads();
-      if (fail) break;
-      const double lkk = A[k * n + k];
-      for (int r = k + 1 + tid; r < n; r += blockDim.x) A[r * n + k] /= lkk;
-      __syncthreads();
-      const int m = n - k - 1;
-      for (int idx = tid; idx < m * m; idx += blockDim.x) {
-        const int r = k + 1 + idx / m, c = k + 1 + idx % m;
-        if (c <= r) A[r * n + c] -= A[r * n + k] * A[c * n + k];
+      const int r = k + 1 + (tid & 63), q = tid >> 6;
+      if (r <= n) {
+        const double l = A[r * P + k] * iv;
+        double* row = A + r * P;
+        const int c1 = r < n ? r : n - 1;
+#pragma unroll 4
+        for (int c = k + 1 + q; c <= c1; c += 2) row[c] -= l * A[c * P + k];
+        if (q == 0) {
+          if (r < n) A[k * P + r] = l;
+          else z[k] = l;
+        }
+        if (tid == 0 && r < n) inv[r] = reciprocal(row[r]);
       }
       __syncthreads();
     }
-    if (!fail) { ok = true; break; }
-    lam *= 10.0;
+    if (!ok) lam *= 10.0;
   }
-  __syncthreads();
   if (!ok) {
-    for (int r = tid; r < n; r += blockDim.x) delta[gp[r]] = 0.0;
+    if (tid < n) delta[gp[tid]] = 0.0;
     if (tid == 0) { atomicCAS(status, 0, AP_ERR_NOT_SPD); lambda[g] = lam; }
     return;
   }
-  // forward and back substitution (one thread: n <= 64)
-  if (tid == 0) {
-    for (int r = 0; r < n; ++r) {
-      double s = jtwr[gp[r]];
-      for (int c = 0; c < r; ++c) s -= A[r * n + c] * y[c];
-      y[r] = s / A[r * n + r];
+  // L^T x = z: x_k is final once the columns past k have been taken out
+  if (warp == 0) {
+    double xa = lane < n ? z[lane] : 0.0, xb = lane + 32 < n ? z[lane + 32] : 0.0;
+    for (int k = n - 1; k > 0; --k) {
+      const double xk = __shfl_sync(0xffffffffu, k < 32 ? xa : xb, k & 31);
+      if (lane < k) xa -= A[lane * P + k] * xk;
+      if (lane + 32 < k) xb -= A[(lane + 32) * P + k] * xk;
     }
-    for (int r = n - 1; r >= 0; --r) {
-      double s = y[r];
-      for (int c = r + 1; c < n; ++c) s -= A[c * n + r] * y[c];
-      y[r] = s / A[r * n + r];
-    }
-    lambda[g] = lam;
+    if (lane < n) delta[gp[lane]] = xa;
+    if (lane + 32 < n) delta[gp[lane + 32]] = xb;
+    if (lane == 0) lambda[g] = lam;
   }
-  __syncthreads();
-  for (int r = tid; r < n; r += blockDim.x) delta[gp[r]] = y[r];
 }
 
 // ---------------------------------------------------------------------------
@@ -836,9 +853,9 @@ void launch_lm_solve(int n_groups, const SolvePlan& sp, const double* vals, cons
                      int max_pcg) {
   if (n_groups <= 0) return;
   if (any_dense) {
-    const size_t sm = (size_t)(2 * max_dense * max_dense + 2 * max_dense) * sizeof(double);
-    chol_kernel<<<n_groups, CHOL_THREADS, sm, st>>>(sp.groups, n_groups, sp.gparams, sp.plocal, sp.row_ptr,
-                                                    sp.col_idx, vals, jtwr, lambda, delta, max_dense, status);
+    const size_t sm = (size_t)((max_dense + 1) * chol_pitch(max_dense) + 3 * max_dense) * sizeof(double);
+    chol_kernel<<<n_groups, CHOL_THREADS, sm, st>>>(sp.groups, sp.gparams, sp.row_ptr, sp.lcol, sp.dpos, vals, jtwr,
+                                                    lambda, delta, max_dense, status);
   }
   if (any_pcg)
     pcg_kernel<<<n_groups, PCG_THREADS, 6 * max_pcg * sizeof(double), st>>>(
@@ -862,78 +879,69 @@ void launch_trial(const double* theta, const double* delta, const double* lo, co
 
 constexpr double LAMBDA_DOWN = 9.0, LAMBDA_UP = 11.0, LAMBDA_MIN = 1e-12, LAMBDA_MAX = 1e12;
 
-// fwd_valid[g] = 1: after this iteration's state copy the group's current
-// source records and w r are in place (the trial's if it accepted, else
-// those of the unchanged theta), and chi2_state holds its chi^2
-__global__ void accept_groups_kernel(const double* chi2_now, const double* chi2_trial, double* lambda,
-                                     double* chi2_state, double* log, int* accepted, int* fwd_valid, int n_groups) {
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= n_groups) return;
-  const double c0 = chi2_now[g], c1 = chi2_trial[g];
-  const int acc = isfinite(c1) && c1 < c0;
-  double lam = lambda[g];
-  lam = acc ? fmax(lam / LAMBDA_DOWN, LAMBDA_MIN) : fmin(lam * LAMBDA_UP, LAMBDA_MAX);
-  lambda[g] = lam;
-  accepted[g] = acc;
-  chi2_state[g] = acc ? c1 : c0;
-  if (fwd_valid) fwd_valid[g] = 1;
-  if (log) {
-    log[4 * g + 0] = c0;
-    log[4 * g + 1] = c1;
-    log[4 * g + 2] = lam;
-    log[4 * g + 3] = acc;
+// Accept or reject, one launch: the first blocks update the groups and the
+// parameters, the others copy an accepted group's trial state (source records,
+// w r) over its current one, a chunk each (16-byte words where both ends are
+// aligned).  Every block decides from the two chi^2 values itself, so nothing in
+// the launch waits for the groups' flags; a chunk is 16 KB, four rounds of loads
+// of its CTA (64 KB chunks in a launch of their own took 11 us on an image of one
+// chunk).
+// fwd_valid[g] = 1: after this launch the group's current source records and w r
+// are in place (the trial's if it accepted, else those of the unchanged theta),
+// and chi2_state holds its chi^2.
+__device__ __forceinline__ bool lm_accepts(const double* chi2_now, const double* chi2_trial, int g) {
+  const double c1 = chi2_trial[g];
+  return isfinite(c1) && c1 < chi2_now[g];
+}
+
+__global__ void __launch_bounds__(256) accept_kernel(const double* __restrict__ chi2_now,
+                                                     const double* __restrict__ chi2_trial, double* lambda,
+                                                     double* chi2_state, double* log, int* fwd_valid, int n_groups,
+                                                     const int* __restrict__ param_group, int n_params, double* theta,
+                                                     const double* __restrict__ trial, int n_head,
+                                                     const StateChunk* __restrict__ chunks) {
+  if ((int)blockIdx.x >= n_head) {
+    const StateChunk ch = chunks[blockIdx.x - n_head];
+    if (!lm_accepts(chi2_now, chi2_trial, ch.group)) return;
+    int done = 0;
+    if ((((uintptr_t)ch.src | (uintptr_t)ch.dst) & 15) == 0) {
+      const int nq = ch.n_words >> 2;
+      const uint4* s4 = reinterpret_cast<const uint4*>(ch.src);
+      uint4* d4 = reinterpret_cast<uint4*>(ch.dst);
+#pragma unroll 4
+      for (int i = threadIdx.x; i < nq; i += 256) d4[i] = __ldg(s4 + i);
+      done = nq << 2;
+    }
+    for (int i = done + threadIdx.x; i < ch.n_words; i += 256) ch.dst[i] = ch.src[i];
+    return;
+  }
+  const int t = blockIdx.x * 256 + threadIdx.x;
+  if (t < n_params) {
+    const int g = param_group[t];
+    if (g >= 0 && lm_accepts(chi2_now, chi2_trial, g)) theta[t] = trial[t];
+  }
+  if (t < n_groups) {
+    const double c0 = chi2_now[t], c1 = chi2_trial[t];
+    const bool acc = lm_accepts(chi2_now, chi2_trial, t);
+    double lam = lambda[t];
+    lam = acc ? fmax(lam / LAMBDA_DOWN, LAMBDA_MIN) : fmin(lam * LAMBDA_UP, LAMBDA_MAX);
+    lambda[t] = lam;
+    chi2_state[t] = acc ? c1 : c0;
+    fwd_valid[t] = 1;
+    log[4 * t + 0] = c0;
+    log[4 * t + 1] = c1;
+    log[4 * t + 2] = lam;
+    log[4 * t + 3] = acc;
   }
 }
 
-__global__ void accept_params_kernel(const int* param_group, int n_params, const int* accepted, double* theta,
-                                     const double* trial) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n_params) return;
-  const int g = param_group[p];
-  if (g >= 0 && accepted[g]) theta[p] = trial[p];
-}
-
-void launch_accept_groups(const double* chi2_now, const double* chi2_trial, double* lambda, double* chi2_state,
-                          double* log, int* accepted, int* fwd_valid, int n_groups, cudaStream_t st) {
-  if (n_groups > 0)
-    accept_groups_kernel<<<(n_groups + 255) / 256, 256, 0, st>>>(chi2_now, chi2_trial, lambda, chi2_state, log,
-                                                                 accepted, fwd_valid, n_groups);
-}
-
-// one CTA per chunk: an accepted group's trial records and w r become its
-// current ones (16-byte words where both ends are aligned)
-__global__ void __launch_bounds__(256) accept_state_kernel(const StateChunk* __restrict__ chunks,
-                                                           const int* __restrict__ accepted) {
-  const StateChunk ch = chunks[blockIdx.x];
-  if (!accepted[ch.group]) return;
-  int done = 0;
-  if ((((uintptr_t)ch.src | (uintptr_t)ch.dst) & 15) == 0) {
-    const int nq = ch.n_words >> 2;
-    const uint4* s4 = reinterpret_cast<const uint4*>(ch.src);
-    uint4* d4 = reinterpret_cast<uint4*>(ch.dst);
-    for (int i = threadIdx.x; i < nq; i += blockDim.x) d4[i] = s4[i];
-    done = nq << 2;
-  }
-  for (int i = done + threadIdx.x; i < ch.n_words; i += blockDim.x) ch.dst[i] = ch.src[i];
-}
-
-void launch_accept_state(const StateChunk* chunks, int n_chunks, const int* accepted, cudaStream_t st) {
-  if (n_chunks > 0) accept_state_kernel<<<n_chunks, 256, 0, st>>>(chunks, accepted);
-}
-
-void launch_accept_params(const int* param_group, int n_params, const int* accepted, double* theta,
-                          const double* trial, cudaStream_t st) {
-  if (n_params > 0)
-    accept_params_kernel<<<(n_params + 255) / 256, 256, 0, st>>>(param_group, n_params, accepted, theta, trial);
-}
-
-__global__ void scale_kernel(const double* in, double* out, double s, int n) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < n) out[p] = s * in[p];
-}
-
-void launch_scale(const double* in, double* out, double s, int n, cudaStream_t st) {
-  if (n > 0) scale_kernel<<<(n + 255) / 256, 256, 0, st>>>(in, out, s, n);
+void launch_accept(const double* chi2_now, const double* chi2_trial, double* lambda, double* chi2_state, double* log,
+                   int* fwd_valid, int n_groups, const int* param_group, int n_params, double* theta,
+                   const double* trial, const StateChunk* chunks, int n_chunks, cudaStream_t st) {
+  const int n_head = (std::max(n_groups, n_params) + 255) / 256;
+  if (n_head + n_chunks > 0)
+    accept_kernel<<<n_head + n_chunks, 256, 0, st>>>(chi2_now, chi2_trial, lambda, chi2_state, log, fwd_valid,
+                                                     n_groups, param_group, n_params, theta, trial, n_head, chunks);
 }
 
 // Pointers carried by value in the kernel's arguments: the launch copies them,
