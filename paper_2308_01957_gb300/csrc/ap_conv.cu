@@ -21,6 +21,8 @@
 // loop issues 16 RY FMAs per RY + 1 shared-memory loads.  Tile variants
 // (threads BX x BY, RY) are picked per problem by timing them (autotuner in
 // ap_api.cu).
+#include <vector>
+
 #include "ap_internal.cuh"
 
 namespace ap {
@@ -48,11 +50,45 @@ template <> struct Vec4<double> {
 
 // variant table: threads BX x BY, rows per thread RY
 struct ConvShape { int bx, by, ry; };
-static const ConvShape kShapes[N_CONV_VARIANTS] = {{16, 16, 4}, {16, 8, 4}, {8, 16, 4}, {16, 16, 2}, {16, 8, 8}, {32, 8, 4},
+// (the first one for small images: a 128^2 image makes 64 CTAs of it, 16 of the
+// next larger one)
+static const ConvShape kShapes[N_CONV_VARIANTS] = {{8, 8, 1}, {16, 8, 4}, {8, 16, 4}, {16, 16, 2}, {16, 8, 8}, {32, 8, 4},
                                                    {16, 8, 2}};
 int conv_tile_w(int v) { return kShapes[v].bx * RX; }
 int conv_tile_h(int v) { return kShapes[v].by * kShapes[v].ry; }
 int conv_threads(int v) { return kShapes[v].bx * kShapes[v].by; }
+
+// The tile's input window and PSF into shared memory by asynchronous copies, all
+// in flight together (through registers every round of the loop waited for its
+// load: 13 of the 17 us of a 128^2 image's correlation).  Outside the input the
+// copies fill zeros.
+template <typename T>
+__device__ __forceinline__ void copy_async(unsigned dst, const T* src, bool in) {
+  if constexpr (sizeof(T) == 4)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(in ? 8 : 0) : "memory");
+}
+template <typename T, int NT>
+__device__ __forceinline__ void load_tile(const T* __restrict__ in, int Hi, int Wi, int in_r0, int in_c0,
+                                          const T* __restrict__ pk, int n_pk, T* s_in, T* s_pk, int SH, int SW) {
+  const int tid = threadIdx.x;
+  const unsigned d_pk = (unsigned)__cvta_generic_to_shared(s_pk), d_in = (unsigned)__cvta_generic_to_shared(s_in);
+  constexpr int V = 16 / sizeof(T);   // PSF rows are whole 16-byte words
+#pragma unroll 2
+  for (int idx = tid * V; idx < n_pk; idx += NT * V)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d_pk + idx * (unsigned)sizeof(T)), "l"(pk + idx)
+                 : "memory");
+#pragma unroll 4
+  for (int idx = tid; idx < SH * SW; idx += NT) {
+    const int r = idx / SW, c = idx - r * SW;
+    const int gr = in_r0 + r, gc = in_c0 + c;
+    const bool inside = gr >= 0 && gr < Hi && gc >= 0 && gc < Wi;
+    copy_async<T>(d_in + idx * (unsigned)sizeof(T), in + (inside ? (size_t)gr * Wi + gc : 0), inside);
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+}
 
 template <typename T, int BX, int BY, int RY>
 __device__ __forceinline__ void corr_tile(const T* __restrict__ in, int Hi, int Wi, int in_r0, int in_c0,
@@ -65,15 +101,7 @@ __device__ __forceinline__ void corr_tile(const T* __restrict__ in, int Hi, int 
   T* s_in = smem;
   T* s_pk = smem + SH * SW;
   const int tid = threadIdx.x;
-  for (int idx = tid; idx < K * K4; idx += NT) s_pk[idx] = pk[idx];
-  for (int idx = tid; idx < SH * SW; idx += NT) {
-    const int r = idx / SW, c = idx - r * SW;
-    const int gr = in_r0 + r, gc = in_c0 + c;
-    T v = (T)0;
-    if (gr >= 0 && gr < Hi && gc >= 0 && gc < Wi) v = in[(size_t)gr * Wi + gc];
-    s_in[idx] = v;
-  }
-  __syncthreads();
+  load_tile<T, NT>(in, Hi, Wi, in_r0, in_c0, pk, K * K4, s_in, s_pk, SH, SW);
   const int lx = tid % BX, ly = tid / BX;
 #pragma unroll
   for (int a = 0; a < RY; ++a)
@@ -119,15 +147,7 @@ __device__ __forceinline__ void corr_tile_nc(const float* __restrict__ in, int H
   float* s_in = smem;
   float* s_pk = smem + SH * SW;
   const int tid = threadIdx.x;
-  for (int idx = tid; idx < K * K4; idx += NT) s_pk[idx] = pk[idx];
-  for (int idx = tid; idx < SH * SW; idx += NT) {
-    const int r = idx / SW, c = idx - r * SW;
-    const int gr = in_r0 + r, gc = in_c0 + c;
-    float v = 0.f;
-    if (gr >= 0 && gr < Hi && gc >= 0 && gc < Wi) v = in[(size_t)gr * Wi + gc];
-    s_in[idx] = v;
-  }
-  __syncthreads();
+  load_tile<float, NT>(in, Hi, Wi, in_r0, in_c0, pk, K * K4, s_in, s_pk, SH, SW);
   const int lx = tid % BX, ly = tid / BX;
 #pragma unroll
   for (int a = 0; a < RY; ++a)
@@ -196,29 +216,45 @@ __global__ void __launch_bounds__(BX * BY) forward_conv_kernel(const ConvWork* _
       for (int b = 0; b < RX; ++b) acc[a][b] = (T)0;
   }
   const int lx = threadIdx.x % BX, ly = threadIdx.x / BX;
-  const T* U = (const T*)im.unc;
+  const T* __restrict__ U = (const T*)im.unc;
+  const float* __restrict__ data = im.data;
+  const float* __restrict__ varp = im.var;
+  const uint8_t* __restrict__ mask = im.mask;
   T* WR = (T*)(trial ? im.wr_trial : im.wr);
+  float* SW = sizeof(T) == 4 && store_sw ? im.sw : nullptr;
   T* M = model_out ? (T*)model_out[w.image] : nullptr;
   // per-pixel residual math in T (float64 is scarce on this GPU); the
   // thread's chi^2 partial of at most RY * 4 terms joins the block sum in
-  // float64
+  // float64.  A row's inputs are all loaded before its first store.
   T c2t = (T)0;
   int bad = 0;
 #pragma unroll
   for (int ry = 0; ry < RY; ++ry) {
     const int oi = w.r0 + ly * RY + ry;
     if (oi >= im.H) break;
+    const int oj0 = w.c0 + lx * RX;
+    const size_t o0 = (size_t)oi * im.W + oj0;
+    T u[RX];
+    float dv[RX], vv[RX];
+    int mk[RX];
 #pragma unroll
     for (int rx = 0; rx < RX; ++rx) {
-      const int oj = w.c0 + lx * RX + rx;
-      if (oj < im.W) {
-        const size_t o = (size_t)oi * im.W + oj;
-        const T m = acc[ry][rx] + U[o];
+      const bool in = oj0 + rx < im.W;
+      u[rx] = in ? __ldg(U + o0 + rx) : (T)0;
+      dv[rx] = in ? __ldg(data + o0 + rx) : 0.f;
+      vv[rx] = in ? __ldg(varp + o0 + rx) : 1.f;
+      mk[rx] = in && mask != nullptr ? (int)__ldg(mask + o0 + rx) : 0;
+    }
+#pragma unroll
+    for (int rx = 0; rx < RX; ++rx) {
+      if (oj0 + rx < im.W) {
+        const size_t o = o0 + rx;
+        const T m = acc[ry][rx] + u[rx];
         if (M) M[o] = m;
-        const T r = (T)im.data[o] - m;
-        const T var = (T)im.var[o];
+        const T r = (T)dv[rx] - m;
+        const T var = (T)vv[rx];
         T wt = (T)0;
-        if (im.mask == nullptr || im.mask[o] == 0) {
+        if (mk[rx] == 0) {
           if (var > (T)0 && var <= Limits<T>::max_finite()) wt = (T)1 / var;
           else bad = 1;
         }
@@ -226,7 +262,7 @@ __global__ void __launch_bounds__(BX * BY) forward_conv_kernel(const ConvWork* _
         c2t += wr * r;
         WR[o] = wr;
         // sqrt(w) for the Jacobian columns (correctly rounded division and root)
-        if (sizeof(T) == 4 && store_sw) im.sw[o] = wt > (T)0 ? 1.0f / sqrtf((float)var) : 0.f;
+        if (SW) SW[o] = wt > (T)0 ? 1.0f / sqrtf((float)var) : 0.f;
       }
     }
   }
@@ -361,7 +397,7 @@ __host__ __device__ constexpr bool fast_shape(int bx, int by, int ry) {
 
 #define AP_CONV_SWITCH(v, CALL, ...)                     \
   switch (v) {                                           \
-    case 0: CALL(16, 16, 4, __VA_ARGS__); break;         \
+    case 0: CALL(8, 8, 1, __VA_ARGS__); break;           \
     case 1: CALL(16, 8, 4, __VA_ARGS__); break;          \
     case 2: CALL(8, 16, 4, __VA_ARGS__); break;          \
     case 3: CALL(16, 16, 2, __VA_ARGS__); break;         \
@@ -439,15 +475,24 @@ static void jc_launch(const JcolWork* work, int n, const SourceDev* srcs, const 
 }
 
 // Launch one kernel per range of work items sharing a PSF chunk count
-// (ranges[k] = {nc, start, count}); nc = 0 runs the generic tile.
+// (ranges[k] = {nc, start, count}); nc = 0 runs the generic tile, and a shape
+// without chunk-count instantiations takes all ranges in one launch.
+static std::vector<ConvRange> launch_ranges(int v, const ConvRange* ranges, int n_ranges) {
+  std::vector<ConvRange> out;
+  for (int k = 0; k < n_ranges; ++k) {
+    if (ranges[k].count <= 0) continue;
+    if (!conv_variant_fast(v) && !out.empty()) out.back().count += ranges[k].count;   // ranges lie one after another
+    else out.push_back(ConvRange{conv_variant_fast(v) ? ranges[k].nc : 0, ranges[k].start, ranges[k].count});
+  }
+  return out;
+}
+
 template <typename T>
 void launch_forward_conv(int v, const ConvWork* work, const ConvRange* ranges, int n_ranges, const ImageDev* imgs,
                          double* chi2_partial, void* const* model_out, const int* skip, int trial, int store_sw,
                          int* status, int kmax, cudaStream_t st) {
-  for (int k = 0; k < n_ranges; ++k) {
-    const ConvRange r = ranges[k];
-    if (r.count <= 0) continue;
-    const int nc = conv_variant_fast(v) ? r.nc : 0;
+  for (const ConvRange& r : launch_ranges(v, ranges, n_ranges)) {
+    const int nc = r.nc;
 #define AP_FWD_NC(NC, BX, BY, RY) fwd_launch<T, BX, BY, RY, NC>(work + r.start, r.count, imgs, chi2_partial + r.start, model_out, skip, trial, store_sw, status, kmax, st)
 #define AP_FWD(BX, BY, RY, dummy) AP_NC_SWITCH(T, nc, AP_FWD_NC, BX, BY, RY)
     AP_CONV_SWITCH(v, AP_FWD, 0)
@@ -459,10 +504,8 @@ void launch_forward_conv(int v, const ConvWork* work, const ConvRange* ranges, i
 template <typename T>
 void launch_adjoint_conv(int v, const ConvWork* work, const ConvRange* ranges, int n_ranges, const ImageDev* imgs,
                          int kmax, cudaStream_t st) {
-  for (int k = 0; k < n_ranges; ++k) {
-    const ConvRange r = ranges[k];
-    if (r.count <= 0) continue;
-    const int nc = conv_variant_fast(v) ? r.nc : 0;
+  for (const ConvRange& r : launch_ranges(v, ranges, n_ranges)) {
+    const int nc = r.nc;
 #define AP_ADJ_NC(NC, BX, BY, RY) adj_launch<T, BX, BY, RY, NC>(work + r.start, r.count, imgs, kmax, st)
 #define AP_ADJ(BX, BY, RY, dummy) AP_NC_SWITCH(T, nc, AP_ADJ_NC, BX, BY, RY)
     AP_CONV_SWITCH(v, AP_ADJ, 0)
@@ -474,10 +517,8 @@ void launch_adjoint_conv(int v, const ConvWork* work, const ConvRange* ranges, i
 template <typename T>
 void launch_jcol(int v, const JcolWork* work, const ConvRange* ranges, int n_ranges, const SourceDev* srcs,
                  const ImageDev* imgs, const T* dbuf, T* jbuf, int kmax, cudaStream_t st) {
-  for (int k = 0; k < n_ranges; ++k) {
-    const ConvRange r = ranges[k];
-    if (r.count <= 0) continue;
-    const int nc = conv_variant_fast(v) ? r.nc : 0;
+  for (const ConvRange& r : launch_ranges(v, ranges, n_ranges)) {
+    const int nc = r.nc;
 #define AP_JC_NC(NC, BX, BY, RY) jc_launch<T, BX, BY, RY, NC>(work + r.start, r.count, srcs, imgs, dbuf, jbuf, kmax, st)
 #define AP_JC(BX, BY, RY, dummy) AP_NC_SWITCH(T, nc, AP_JC_NC, BX, BY, RY)
     AP_CONV_SWITCH(v, AP_JC, 0)
