@@ -371,7 +371,7 @@ struct GroupDev {
 // chunks of DIST_WCHUNK entries (more for rows that would otherwise have more
 // than DIST_MAX_PARTS chunks)
 constexpr int DIST_CHUNK = 16;
-constexpr int DIST_WARP_ROW = 64;
+constexpr int DIST_WARP_ROW = 512;   // (64 and 256 were slower on every fit timed but the 12-image one, within 5 %)
 constexpr int DIST_WCHUNK = 128;
 constexpr int DIST_MAX_PARTS = 16;
 

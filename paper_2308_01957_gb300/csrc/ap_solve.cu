@@ -369,13 +369,19 @@ __global__ void __launch_bounds__(PCG_THREADS) pcg_kernel(const GroupDev* __rest
 // its shared memory.  The SpMV is cut into chunks that any CTA may compute:
 // rows of up to DIST_WARP_ROW entries into thread chunks of DIST_CHUNK
 // entries, longer rows (the sky parameters couple to everything) into warp
-// chunks of DIST_WCHUNK entries, so that no row has more than a few partials
-// to add.  In a cluster, u is broadcast into every CTA's shared memory and
+// chunks of DIST_WCHUNK entries, so that no row has more than a few tens of
+// partials to add.  What an iteration waits for is the count of float64 warp
+// instructions (profiled on a 112-parameter fit: the float64 pipe 55 % busy,
+// 600 of them per SM and iteration): a thread chunk costs 16 for 512 entries
+// where a warp chunk costs 10 for 128.  The first chunk of every thread stays in
+// registers over the iterations.  21 iterations of the 953-parameter field 298 ->
+// 211 us, 43 of 16 overlapping galaxies 413 -> 299 us, 82 grid-wide ones of the
+// 1536^2 crowded field 2.10 -> 1.84 ms.  In a cluster, u is broadcast into every CTA's shared memory and
 // each chunk partial is stored straight into its row owner's shared memory
 // (distributed shared memory); grid-wide, both go through global memory.
-// Reductions: every CTA publishes its block totals to slot[parity][rank];
-// after the barrier every CTA adds the slots in rank order, so all CTAs hold
-// the same bits and take the same branches.
+// Reductions: every CTA publishes its totals to its rank's slots; after the
+// barrier every CTA adds the slots in rank order, so all CTAs hold the same
+// bits and take the same branches.
 // ---------------------------------------------------------------------------
 constexpr int DIST_THREADS = 256;
 
@@ -400,81 +406,63 @@ struct ClusterBarrier {
   __device__ T* at(T* p, int q) const { return cg::this_cluster().map_shared_rank(p, q); }
 };
 
-// CTA totals of NV <= 3 values (value 0 is a max when max0); every lane of
-// warp 0 ends with them.  The tree joining the warp partials is only as wide
-// as there are warps (every float64 instruction is costly on this part).
-// red[] holds 3 x 32 + 3 doubles.
-template <int NV>
-__device__ void cta_reduce(double v[3], bool max0, double* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nw = (blockDim.x + 31) >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double t = __shfl_xor_sync(0xffffffffu, v[k], o);
-      v[k] = (k == 0 && max0) ? fmax(v[k], t) : v[k] + t;
-    }
-  __syncthreads();
-  if (lane == 0)
-    for (int k = 0; k < NV; ++k) red[warp * 3 + k] = v[k];
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      v[k] = lane < nw ? red[lane * 3 + k] : 0.0;
-      for (int o = 16; o > 0; o >>= 1) {
-        if (o >= nw) continue;   // uniform: the lanes past nw hold zeros
-        const double t = __shfl_xor_sync(0xffffffffu, v[k], o);
-        v[k] = (k == 0 && max0) ? fmax(v[k], t) : v[k] + t;
-      }
-      // after the trimmed tree only the lanes below nw hold the total: lane
-      // 0's copy goes to every lane (a cluster publishes from lanes 0..nct-1)
-      v[k] = __shfl_sync(0xffffffffu, v[k], 0);
-    }
-  }
-}
-
-// publish the CTA totals into slot[par][rank] (every CTA's copy in a
-// cluster, the one global copy otherwise), wait at the barrier, add the slots
-// in rank order; every thread returns the same NV values
+// Totals over all CTAs of NV <= 3 values (value 0 is a max when max0).  A warp-wide
+// float64 addition holds this part's one float64 pipe per SM for some 17 clocks
+// whatever its lanes do, and they were what an iteration waited for, so the totals
+// take as few of them as they can: every thread leaves its values in shared memory,
+// warp k adds value k (8 terms per lane, then one tree) and publishes it to
+// slot[par][k][rank] -- every CTA's copy in a cluster, the one global copy otherwise
+// -- waits at the barrier and adds the slots in rank order (17 additions per value;
+// a tree in every warp took 47).  Every thread returns the same NV values.
+// red[] holds 3 DIST_THREADS + 3 doubles.
 template <int NV, class Bar>
 __device__ void dist_reduce(const Bar& bar, double v[3], bool max0, double* slots, int& par, double* red) {
   const int nct = bar.size(), rank = bar.rank();
-  cta_reduce<NV>(v, max0, red);
-  double* sp = slots + (size_t)par * nct * 4;
-  if (Bar::kCluster) {
-    // every lane of warp 0 holds the totals; lane q stores them into CTA q
-    if (threadIdx.x < nct) {
-      double* dst = bar.at(sp, threadIdx.x) + rank * 4;
-      for (int k = 0; k < NV; ++k) dst[k] = v[k];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) red[k * DIST_THREADS + threadIdx.x] = v[k];
+  __syncthreads();
+  const bool mx = warp == 0 && max0;
+  auto join = [&](double x, double y) { return mx ? fmax(x, y) : x + y; };
+  double* sp = slots + (size_t)(par * 3 + warp) * nct;
+  if (warp < NV) {
+    const double* r = red + warp * DIST_THREADS + lane;
+    double x = join(r[0], r[32]), y = join(r[64], r[96]), z = join(r[128], r[160]), w = join(r[192], r[224]);
+    x = join(join(x, y), join(z, w));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = join(x, __shfl_xor_sync(0xffffffffu, x, o));
+    if (Bar::kCluster) {
+      if (lane < nct) bar.at(sp, lane)[rank] = x;
+    } else if (lane == 0) {
+      sp[rank] = x;
     }
-  } else if (threadIdx.x == 0) {
-    for (int k = 0; k < NV; ++k) sp[rank * 4 + k] = v[k];
   }
   bar.sync();
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    double s[3] = {0.0, 0.0, 0.0};
-    for (int q = lane; q < nct; q += 32)
-      for (int k = 0; k < NV; ++k) {
-        const double t = Bar::kCluster ? sp[q * 4 + k] : __ldcg(sp + q * 4 + k);
-        s[k] = (k == 0 && max0) ? fmax(s[k], t) : s[k] + t;
-      }
+  if (warp < NV) {
+    double x = 0.0;   // (the max is over non-negative values)
+    if constexpr (Bar::kCluster) {
+      x = lane < nct ? sp[lane] : 0.0;
+    } else {
+      for (int q0 = lane; q0 < nct; q0 += 320) {   // ten slots per lane in flight
+        double t[10];
 #pragma unroll
-    for (int k = 0; k < NV; ++k)
-      for (int o = 16; o > 0; o >>= 1) {
-        if (o >= nct) continue;   // uniform: the lanes past nct hold zeros
-        const double t = __shfl_xor_sync(0xffffffffu, s[k], o);
-        s[k] = (k == 0 && max0) ? fmax(s[k], t) : s[k] + t;
+        for (int j = 0; j < 10; ++j) t[j] = q0 + 32 * j < nct ? __ldcg(sp + q0 + 32 * j) : 0.0;
+#pragma unroll
+        for (int j = 0; j < 10; ++j) x = join(x, t[j]);
       }
-    if (lane == 0)   // lane 0 holds the complete sum
-      for (int k = 0; k < NV; ++k) red[96 + k] = s[k];
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      if (o >= nct) continue;   // uniform: the lanes past nct hold zeros
+      x = join(x, __shfl_xor_sync(0xffffffffu, x, o));
+    }
+    if (lane == 0) red[3 * DIST_THREADS + warp] = x;
   }
   __syncthreads();
-  for (int k = 0; k < NV; ++k) v[k] = red[96 + k];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) v[k] = red[3 * DIST_THREADS + k];
   par ^= 1;
 }
+static_assert(DIST_THREADS == 256, "eight terms per lane");
 
 // read u: the CTA's own copy in a cluster, global memory (L2) otherwise
 template <bool CL>
@@ -535,7 +523,7 @@ __global__ void __launch_bounds__(DIST_THREADS, 2) pcg_dist_kernel(int g_fixed, 
   constexpr bool CL = Bar::kCluster;
   const Bar bar;
   extern __shared__ double sm[];
-  __shared__ double red[3 * 32 + 3];
+  __shared__ double red[3 * DIST_THREADS + 3];
   const int nct = bar.size(), rank = bar.rank();
   const int tid = threadIdx.x, lane = tid & 31;
   const int g = CL ? glist[bar.unit()] : g_fixed;
@@ -548,7 +536,7 @@ __global__ void __launch_bounds__(DIST_THREADS, 2) pcg_dist_kernel(int g_fixed, 
   const int P0 = dp.row[G.p0 + R0];   // first chunk partial of the owned rows
   // shared memory: [slots (cluster)] | x r p s D [nr] | block inverses [nb] | u [nu] | partials [np] (cluster)
   double* slots = CL ? sm : gslots;
-  double* X = sm + (CL ? 8 * nct : 0);
+  double* X = sm + (CL ? 6 * nct : 0);
   double* Rv = X + sz.nr;
   double* P = Rv + sz.nr;
   double* S = P + sz.nr;
@@ -558,7 +546,9 @@ __global__ void __launch_bounds__(DIST_THREADS, 2) pcg_dist_kernel(int g_fixed, 
   double* PART = U + sz.nu;                   // cluster: partials of the owned rows
   double* gu = work + (int64_t)6 * G.p0;      // grid: u over the whole group, in global memory
   const double* ug = CL ? U : gu;             // where the SpMV gathers u from
-  const int first = rank + nct * tid, stride = nct * (int)blockDim.x;
+  // thread chunks go to the CTA's threads from the last one down, warp chunks to its
+  // warps from the first one up: the warps with warp chunks get thread chunks last
+  const int first = rank + nct * ((int)blockDim.x - 1 - tid), stride = nct * (int)blockDim.x;
   const int wfirst = rank + nct * (tid >> 5), wstride = nct * (int)(blockDim.x >> 5);
   int par = 0;
   if (CL) bar.sync();   // every CTA of the cluster is running before any remote store
@@ -595,6 +585,23 @@ __global__ void __launch_bounds__(DIST_THREADS, 2) pcg_dist_kernel(int g_fixed, 
   const int team = tid / PCG_BLK, tl = tid % PCG_BLK, tbase = lane & ~(PCG_BLK - 1);
   const int nteam = blockDim.x / PCG_BLK;
   const int nrounds = (b1 - b0 + nteam - 1) / nteam;
+  // the chunks of the first round's row
+  int pc0 = 0, pc1 = 0;
+  if (b0 + team < b1 && tl < bp[b0 + team + 1] - bp[b0 + team]) {
+    pc0 = dp.row[G.p0 + bp[b0 + team] + tl];
+    pc1 = dp.row[G.p0 + bp[b0 + team] + tl + 1];
+  }
+  // the thread's first chunk stays in registers over all iterations
+  double kv[DIST_CHUNK];
+  int kc[DIST_CHUNK];
+  const int kid = tb + first < te ? dp.tlist[tb + first] : -1;
+  const int64_t ke0 = kid >= 0 ? dp.e0[kid] : 0, ke1 = kid >= 0 ? dp.e1[kid] : 0;
+#pragma unroll
+  for (int j = 0; j < DIST_CHUNK; ++j) {
+    const bool in = ke0 + j < ke1;
+    kv[j] = in ? vals[ke0 + j] : 0.0;
+    kc[j] = in ? dp.lcol[ke0 + j] : -1;
+  }
 
   for (int attempt = 0; attempt <= LM_RETRIES && !ok; ++attempt) {
     double fail = 0.0, gam = 0.0, dd = 0.0;
@@ -684,12 +691,23 @@ __global__ void __launch_bounds__(DIST_THREADS, 2) pcg_dist_kernel(int g_fixed, 
           del += ld_u<CL>(ug, dp.lrow[c]) * sv;
         }
       }
-      for (int k = tb + first; k < te; k += stride) {
-        const int c = dp.tlist[k];
-        const double sv = dist_tchunk<CL>(vals, dp.lcol, ug, dp.e0[c], dp.e1[c]);
+      auto put = [&](int c, double sv) {   // a chunk's sum to its row's owner
         if (CL) bar.at(PART, dp.owner[c])[dp.dst[c]] = sv;
         else dp.part[c] = sv;
         del += ld_u<CL>(ug, dp.lrow[c]) * sv;
+      };
+      if (kid >= 0) {
+        double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+        for (int j = 0; j < DIST_CHUNK; j += 2) {
+          if (kc[j] >= 0) a0 += kv[j] * ld_u<CL>(ug, kc[j]);
+          if (kc[j + 1] >= 0) a1 += kv[j + 1] * ld_u<CL>(ug, kc[j + 1]);
+        }
+        put(kid, a0 + a1);
+      }
+      for (int k = tb + first + stride; k < te; k += stride) {
+        const int c = dp.tlist[k];
+        put(c, dist_tchunk<CL>(vals, dp.lcol, ug, dp.e0[c], dp.e1[c]));
       }
       v[0] = del;
       dist_reduce<1>(bar, v, false, slots, par, red);
@@ -707,15 +725,21 @@ __global__ void __launch_bounds__(DIST_THREADS, 2) pcg_dist_kernel(int g_fixed, 
         double rr = 0.0;
         if (row) {
           const int i = s0 + tl;
-          const int c0 = dp.row[G.p0 + i], c1 = dp.row[G.p0 + i + 1];
+          const int c0 = rd == 0 ? pc0 : dp.row[G.p0 + i], c1 = rd == 0 ? pc1 : dp.row[G.p0 + i + 1];
           const double ui = own_u(i);
           double w0 = lam * Dv[l] * ui, w1 = 0.0;
-          int ch = c0;
-          for (; ch + 1 < c1; ch += 2) {
-            w0 += CL ? PART[ch - P0] : __ldcg(dp.part + ch);
-            w1 += CL ? PART[ch + 1 - P0] : __ldcg(dp.part + ch + 1);
+          constexpr int NP = CL ? 4 : 8;
+          for (int ch = c0; ch < c1; ch += NP) {   // NP partials in flight
+            double t[NP];
+#pragma unroll
+            for (int q = 0; q < NP; ++q) t[q] = ch + q < c1 ? (CL ? PART[ch + q - P0] : __ldcg(dp.part + ch + q)) : 0.0;
+#pragma unroll
+            for (int q = 0; q < NP; q += 2)
+              if (ch + q < c1) {
+                w0 += t[q];
+                w1 += t[q + 1];
+              }
           }
-          if (ch < c1) w0 += CL ? PART[ch - P0] : __ldcg(dp.part + ch);
           const double pi = ui + beta * P[l];
           const double si = (w0 + w1) + beta * S[l];
           P[l] = pi;
@@ -768,7 +792,7 @@ __global__ void __launch_bounds__(DIST_THREADS, 2) pcg_dist_kernel(int g_fixed, 
 }
 
 size_t dist_smem_bytes(const DistSmem& sz, int nct, bool cluster) {
-  return sizeof(double) * ((cluster ? (size_t)8 * nct : 0) + 5 * (size_t)sz.nr + (size_t)sz.nb + sz.nu + sz.np);
+  return sizeof(double) * ((cluster ? (size_t)6 * nct : 0) + 5 * (size_t)sz.nr + (size_t)sz.nb + sz.nu + sz.np);
 }
 
 int grid_pcg_blocks(int device, size_t smem) {
