@@ -55,8 +55,8 @@ def _ptr(t: Optional[torch.Tensor]):
 
 
 def _stream(stream) -> Optional[int]:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:   # the current stream's handle, without making a Stream object of it
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
 
 
@@ -139,7 +139,10 @@ class Context:
         self._pg_dev = torch.as_tensor(self.param_group.astype(np.int64), device=self.device)
 
     def _theta(self, theta) -> torch.Tensor:
-        t = torch.as_tensor(theta, dtype=torch.float64, device=self.device).contiguous()
+        if isinstance(theta, torch.Tensor) and theta.dtype is torch.float64 and theta.device == self.device:
+            t = theta.contiguous()
+        else:
+            t = torch.as_tensor(theta, dtype=torch.float64, device=self.device).contiguous()
         if t.numel() != self.n_params:
             raise ValueError(f"theta has {t.numel()} entries, problem has {self.n_params}")
         return t

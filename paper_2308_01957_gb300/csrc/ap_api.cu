@@ -142,6 +142,8 @@ struct ap_ctx {
   void** d_model_ptrs = nullptr;
   int64_t iterations = 0;
   bool lm_started = false;   // ap_lm_iterate has run since the problem was set
+  bool fwd_flags_set = false;   // LM iterations have set d_fwd_valid since it was last cleared
+  bool fwd_flags_captured = false;   // iterations were captured by the caller: a replay may set it any time
   // CUDA graph of one LM iteration
   cudaGraphExec_t lm_exec = nullptr;
   cudaGraph_t lm_graph = nullptr;
@@ -258,6 +260,7 @@ void free_problem(ap_ctx* c) {
   c->jcol_ms_direct = c->jcol_ms_fft = -1.0;
   c->have_problem = false;
   c->lm_started = false;
+  c->fwd_flags_set = c->fwd_flags_captured = false;
   c->have_adapt = false;
   c->adapt = AdaptPlan{};
   c->n_asamples = 0;
@@ -294,17 +297,40 @@ void param_bounds(const std::vector<SourceDev>& srcs, int n_params, std::vector<
   }
 }
 
+// the float64 gathers of what was asked for
+void gather(ap_ctx* c, double* chi2_out, double* grad_out, double* jtwr_out, const int* skip, cudaStream_t st) {
+  launch_gather(GatherPlan{c->d_chi2_partial, c->d_grp_ptr, c->d_grp_idx, chi2_out ? c->n_groups : 0, chi2_out, skip,
+                           c->d_chi2_state, c->d_grad_partial, c->d_gc_ptr, c->d_gc_idx, grad_out ? c->n_params : 0,
+                           grad_out, jtwr_out},
+                st);
+}
+
+// the caller's model pointers as a kernel argument, or through the device table
+ModelOut model_out_of(ap_ctx* c, void* const* model, cudaStream_t st) {
+  ModelOut m;
+  if (!model) return m;
+  if (c->n_img <= MODEL_OUT_MAX) {
+    m.n = c->n_img;
+    std::copy(model, model + c->n_img, m.p);
+  } else {
+    launch_store_ptrs(model, c->n_img, c->d_model_ptrs, st);
+    m.table = c->d_model_ptrs;
+  }
+  return m;
+}
+
 // skip (device, per group, nullable): groups whose source records, w r and
 // chi^2 (d_chi2_state) at theta are already in place keep them; the gradient
 // and everything after it run for every group.  trial: the forward state goes
 // to the trial buffers (d_par_trial, wr_trial), leaving the current point's.
 template <typename T>
 int do_eval(ap_ctx* c, const double* theta, double* chi2_out, double* grad_out, double* jtwr_out,
-            void* const* model_ptrs_dev, const int* skip, bool trial, cudaStream_t st) {
+            const ModelOut& model_out, const int* skip, bool trial, cudaStream_t st) {
   const bool want_D = jtwr_out != nullptr;
   SrcPar<T>* par = (SrcPar<T>*)(trial ? c->d_par_trial : c->d_par);
-  c->launches_last_eval = (c->n_src > 0) + (c->n_rwork > 0) + (c->n_fwork > 0) + (chi2_out && c->n_groups > 0) +
-                          (grad_out ? (c->n_awork > 0) + (c->n_rwork > 0) + (c->n_params > 0) : 0);
+  c->launches_last_eval = (c->n_src > 0) + (c->n_rwork > 0) + (c->n_fwork > 0) +
+                          ((chi2_out && c->n_groups > 0) || (grad_out && c->n_params > 0)) +
+                          (grad_out ? (c->n_awork > 0) + (c->n_rwork > 0) : 0);
   {
     Bracket b(c, st, "prepare");
     launch_prepare<T>(c->d_srcs, c->d_imgs, c->n_src, theta, par, skip, c->d_status, st);
@@ -322,13 +348,8 @@ int do_eval(ap_ctx* c, const double* theta, double* chi2_out, double* grad_out, 
   {
     Bracket b(c, st, "forward_conv_chi2");
     launch_forward_conv<T>(c->conv_variant, c->d_fwork, c->frange.data(), (int)c->frange.size(), c->d_imgs,
-                           c->d_chi2_partial, model_ptrs_dev, skip, trial ? 1 : 0, want_D ? 1 : 0, c->d_status,
+                           c->d_chi2_partial, model_out, skip, trial ? 1 : 0, want_D ? 1 : 0, c->d_status,
                            c->Kmax, st);
-  }
-  if (chi2_out) {
-    Bracket b(c, st, "chi2_gather");
-    launch_sum_groups(c->d_chi2_partial, c->d_grp_ptr, c->d_grp_idx, c->n_groups, chi2_out, 1.0, skip,
-                      c->d_chi2_state, st);
   }
   if (grad_out) {
     {
@@ -346,19 +367,17 @@ int do_eval(ap_ctx* c, const double* theta, double* chi2_out, double* grad_out, 
                                (const SrcPar<T>*)c->d_par, c->d_imgs, c->d_grad_partial,
                                want_D ? (T*)c->d_dbuf : nullptr, want_D && !c->f64 ? (T*)c->d_jbuf : nullptr, st);
     }
-    {
-      Bracket b(c, st, "grad_gather");
-      launch_sum_contrib(c->d_grad_partial, c->d_gc_ptr, c->d_gc_idx, c->n_params, grad_out, -2.0, jtwr_out, st);
-    }
   }
+  Bracket b(c, st, "gather");
+  gather(c, chi2_out, grad_out, jtwr_out, skip, st);
   return AP_OK;
 }
 
 // jtwr_out (nullable, with grad_out): J^T W r, and the derivative images are kept
 int eval_any(ap_ctx* c, const double* theta, double* chi2_out, double* grad_out, double* jtwr_out,
-             void* const* model_ptrs_dev, cudaStream_t st, const int* skip = nullptr, bool trial = false) {
-  return c->f64 ? do_eval<double>(c, theta, chi2_out, grad_out, jtwr_out, model_ptrs_dev, skip, trial, st)
-                : do_eval<float>(c, theta, chi2_out, grad_out, jtwr_out, model_ptrs_dev, skip, trial, st);
+             const ModelOut& model_out, cudaStream_t st, const int* skip = nullptr, bool trial = false) {
+  return c->f64 ? do_eval<double>(c, theta, chi2_out, grad_out, jtwr_out, model_out, skip, trial, st)
+                : do_eval<float>(c, theta, chi2_out, grad_out, jtwr_out, model_out, skip, trial, st);
 }
 
 void launch_jcol_fft_all(ap_ctx* c, cudaStream_t st) {
@@ -381,7 +400,7 @@ void launch_jcol_fft_all(ap_ctx* c, cudaStream_t st) {
 }
 
 int normal_eq_any(ap_ctx* c, const double* theta, double* jtwr_out, cudaStream_t st, const int* skip = nullptr) {
-  int rc = eval_any(c, theta, c->d_chi2, c->d_grad, jtwr_out, nullptr, st, skip);
+  int rc = eval_any(c, theta, c->d_chi2, c->d_grad, jtwr_out, ModelOut{}, st, skip);
   if (rc) return rc;
   cudaMemsetAsync(c->d_vals, 0, (size_t)std::max<int64_t>(c->nnz, 1) * sizeof(double), st);
   {
@@ -440,7 +459,7 @@ int lm_iteration(ap_ctx* c, cudaStream_t st) {
     Bracket b(c, st, "lm_trial");
     launch_trial(c->d_theta, c->d_delta, c->d_lo, c->d_hi, c->d_trial, c->n_params, st);
   }
-  rc = eval_any(c, c->d_trial, c->d_chi2_trial, nullptr, nullptr, nullptr, st, nullptr, true);
+  rc = eval_any(c, c->d_trial, c->d_chi2_trial, nullptr, nullptr, ModelOut{}, st, nullptr, true);
   if (rc) return rc;
   {
     Bracket b(c, st, "lm_accept");
@@ -452,7 +471,19 @@ int lm_iteration(ap_ctx* c, cudaStream_t st) {
 
 // Evaluations outside the LM iteration overwrite the forward buffers: the
 // next LM iteration must evaluate every group at theta.
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;   // (the legacy stream beside a capture elsewhere: as if capturing)
+}
+
+// Nothing to clear if no LM iteration has run since the last time.  A captured
+// call always clears, as its graph may be replayed after an iteration, and so does
+// every call once iterations have been captured.
 int drop_lm_reuse(ap_ctx* c, cudaStream_t st) {
+  if (!c->fwd_flags_set && !c->fwd_flags_captured && !capturing(st)) return AP_OK;
+  c->fwd_flags_set = false;
   CUDA_TRY(c, cudaMemsetAsync(c->d_fwd_valid, 0, (size_t)std::max(c->n_groups, 1) * sizeof(int), st));
   return AP_OK;
 }
@@ -550,7 +581,7 @@ int build_shift(ap_ctx* c) {
 }
 
 template <typename T>
-void eval_shifted(ap_ctx* c, const double* theta, int method, double* chi2_out, bool model_out, cudaStream_t st) {
+void eval_shifted(ap_ctx* c, const double* theta, int method, double* chi2_out, const ModelOut& model_out, cudaStream_t st) {
   SrcPar<T>* par = (SrcPar<T>*)c->d_par;
   {
     Bracket b(c, st, "prepare");
@@ -568,18 +599,17 @@ void eval_shifted(ap_ctx* c, const double* theta, int method, double* chi2_out, 
   {
     Bracket b(c, st, "forward_conv_chi2");
     launch_forward_conv<T>(c->conv_variant, c->d_fwork, c->frange.data(), (int)c->frange.size(), c->d_imgs,
-                           c->d_chi2_partial, model_out ? c->d_model_ptrs : nullptr, nullptr, 0, 0, c->d_status,
+                           c->d_chi2_partial, model_out, nullptr, 0, 0, c->d_status,
                            c->Kmax, st);
   }
   if (chi2_out) {
-    Bracket b(c, st, "chi2_gather");
-    launch_sum_groups(c->d_chi2_partial, c->d_grp_ptr, c->d_grp_idx, c->n_groups, chi2_out, 1.0, nullptr, nullptr,
-                      st);
+    Bracket b(c, st, "gather");
+    gather(c, chi2_out, nullptr, nullptr, nullptr, st);
   }
 }
 
 template <typename T>
-void eval_adaptive(ap_ctx* c, const double* theta, double tol, double* chi2_out, bool model_out, cudaStream_t st) {
+void eval_adaptive(ap_ctx* c, const double* theta, double tol, double* chi2_out, const ModelOut& model_out, cudaStream_t st) {
   SrcPar<T>* par = (SrcPar<T>*)c->d_par;
   {
     Bracket b(c, st, "prepare");
@@ -601,13 +631,12 @@ void eval_adaptive(ap_ctx* c, const double* theta, double tol, double* chi2_out,
   {
     Bracket b(c, st, "forward_conv_chi2");
     launch_forward_conv<T>(c->conv_variant, c->d_fwork, c->frange.data(), (int)c->frange.size(), c->d_imgs,
-                           c->d_chi2_partial, model_out ? c->d_model_ptrs : nullptr, nullptr, 0, 0, c->d_status,
+                           c->d_chi2_partial, model_out, nullptr, 0, 0, c->d_status,
                            c->Kmax, st);
   }
   if (chi2_out) {
-    Bracket b(c, st, "chi2_gather");
-    launch_sum_groups(c->d_chi2_partial, c->d_grp_ptr, c->d_grp_idx, c->n_groups, chi2_out, 1.0, nullptr, nullptr,
-                      st);
+    Bracket b(c, st, "gather");
+    gather(c, chi2_out, nullptr, nullptr, nullptr, st);
   }
 }
 
@@ -616,6 +645,8 @@ void eval_adaptive(ap_ctx* c, const double* theta, double tol, double* chi2_out,
 // caller's buffers
 int lm_run(ap_ctx* c, double* theta, double* lambda, double* chi2, int n_iter, double* log_host, cudaStream_t st) {
   const size_t P = (size_t)c->n_params, G = (size_t)c->n_groups;
+  if (n_iter > 0) c->fwd_flags_set = true;
+  if (capturing(st)) c->fwd_flags_captured = true;
   if (c->timing) {
     // timed mode: the same launch sequence without the graph, every kernel
     // bracketed by events
@@ -666,7 +697,7 @@ int lm_run(ap_ctx* c, double* theta, double* lambda, double* chi2, int n_iter, d
     if (n_iter > 0) {
       CUDA_TRY(c, cudaMemcpyAsync(chi2, c->d_chi2_state, G * sizeof(double), cudaMemcpyDeviceToDevice, st));
     } else {
-      int rc = eval_any(c, c->d_theta, chi2, nullptr, nullptr, nullptr, st);
+      int rc = eval_any(c, c->d_theta, chi2, nullptr, nullptr, ModelOut{}, st);
       if (rc) return rc;
       if ((rc = drop_lm_reuse(c, st))) return rc;
     }
@@ -1754,11 +1785,11 @@ int ap_set_problem(ap_ctx* c, const ap_image_desc* imgs, int n_img, const ap_sou
         const auto& fr = c->v_frange[v];
         const auto& ar = c->v_arange[v];
         if (f64) {
-          launch_forward_conv<double>(v, c->v_fwork[v], fr.data(), (int)fr.size(), c->d_imgs, c->d_chi2_partial, nullptr,
+          launch_forward_conv<double>(v, c->v_fwork[v], fr.data(), (int)fr.size(), c->d_imgs, c->d_chi2_partial, ModelOut{},
                                       nullptr, 0, 0, c->d_status, Kmax, st);
           launch_adjoint_conv<double>(v, c->v_awork[v], ar.data(), (int)ar.size(), c->d_imgs, Kmax, st);
         } else {
-          launch_forward_conv<float>(v, c->v_fwork[v], fr.data(), (int)fr.size(), c->d_imgs, c->d_chi2_partial, nullptr,
+          launch_forward_conv<float>(v, c->v_fwork[v], fr.data(), (int)fr.size(), c->d_imgs, c->d_chi2_partial, ModelOut{},
                                      nullptr, 0, 0, c->d_status, Kmax, st);
           launch_adjoint_conv<float>(v, c->v_awork[v], ar.data(), (int)ar.size(), c->d_imgs, Kmax, st);
         }
@@ -1922,13 +1953,13 @@ int ap_eval_adaptive(ap_ctx* c, const double* theta, double tol, double* chi2, v
   int rc = build_adaptive(c);
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
-  if (model_dev) launch_store_ptrs(model_dev, c->n_img, c->d_model_ptrs, st);
+  const ModelOut mo = model_out_of(c, model_dev, st);
   CUDA_TRY(c, cudaMemsetAsync(c->adapt.n_list, 0, sizeof(int), st));
   CUDA_TRY(c, cudaMemsetAsync(c->adapt.counts, 0, ADAPT_COUNTS * sizeof(unsigned long long), st));
   if (c->f64)
-    eval_adaptive<double>(c, theta, tol, chi2, model_dev != nullptr, st);
+    eval_adaptive<double>(c, theta, tol, chi2, mo, st);
   else
-    eval_adaptive<float>(c, theta, tol, chi2, model_dev != nullptr, st);
+    eval_adaptive<float>(c, theta, tol, chi2, mo, st);
   if (levels_dev && c->n_asamples > 0)
     CUDA_TRY(c, cudaMemcpyAsync(levels_dev, c->adapt.level, (size_t)c->n_asamples, cudaMemcpyDeviceToDevice, st));
   if ((rc = drop_lm_reuse(c, st))) return rc;
@@ -1950,11 +1981,11 @@ int ap_eval_shifted(ap_ctx* c, const double* theta, int method, double* chi2, vo
   int rc = build_shift(c);
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
-  if (model_dev) launch_store_ptrs(model_dev, c->n_img, c->d_model_ptrs, st);
+  const ModelOut mo = model_out_of(c, model_dev, st);
   if (c->f64)
-    eval_shifted<double>(c, theta, method, chi2, model_dev != nullptr, st);
+    eval_shifted<double>(c, theta, method, chi2, mo, st);
   else
-    eval_shifted<float>(c, theta, method, chi2, model_dev != nullptr, st);
+    eval_shifted<float>(c, theta, method, chi2, mo, st);
   if ((rc = drop_lm_reuse(c, st))) return rc;
   CUDA_TRY(c, cudaGetLastError());
   return AP_OK;
@@ -1965,8 +1996,7 @@ int ap_render(ap_ctx* c, const double* theta, void* const* model_dev, void* stre
   if (!c->have_problem) return fail(c, AP_ERR_STATE, "no problem set");
   cudaSetDevice(c->opt.device);
   cudaStream_t st = (cudaStream_t)stream;
-  launch_store_ptrs(model_dev, c->n_img, c->d_model_ptrs, st);
-  int rc = eval_any(c, theta, nullptr, nullptr, nullptr, c->d_model_ptrs, st);
+  int rc = eval_any(c, theta, nullptr, nullptr, nullptr, model_out_of(c, model_dev, st), st);
   if (rc) return rc;
   if ((rc = drop_lm_reuse(c, st))) return rc;
   CUDA_TRY(c, cudaGetLastError());
@@ -1977,7 +2007,7 @@ int ap_eval(ap_ctx* c, const double* theta, double* chi2, double* grad, void* st
   if (!c || !theta || !chi2) return AP_ERR_ARG;
   if (!c->have_problem) return fail(c, AP_ERR_STATE, "no problem set");
   cudaStream_t st = (cudaStream_t)stream;
-  int rc = eval_any(c, theta, chi2, grad, nullptr, nullptr, st);
+  int rc = eval_any(c, theta, chi2, grad, nullptr, ModelOut{}, st);
   if (rc) return rc;
   if ((rc = drop_lm_reuse(c, st))) return rc;
   CUDA_TRY(c, cudaGetLastError());

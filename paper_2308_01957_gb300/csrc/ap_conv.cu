@@ -196,7 +196,7 @@ template <typename T, int BX, int BY, int RY, int NC>
 __global__ void __launch_bounds__(BX * BY) forward_conv_kernel(const ConvWork* __restrict__ work,
                                                                const ImageDev* __restrict__ imgs,
                                                                double* __restrict__ chi2_partial,
-                                                               void* const* __restrict__ model_out,
+                                                               const __grid_constant__ ModelOut model_out,
                                                                const int* __restrict__ skip, int trial,
                                                                int store_sw, int* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(BX * BY) forward_conv_kernel(const ConvWork* _
   const uint8_t* __restrict__ mask = im.mask;
   T* WR = (T*)(trial ? im.wr_trial : im.wr);
   float* SW = sizeof(T) == 4 && store_sw ? im.sw : nullptr;
-  T* M = model_out ? (T*)model_out[w.image] : nullptr;
+  T* M = (T*)(model_out.n > 0 ? model_out.p[w.image] : model_out.table ? model_out.table[w.image] : nullptr);
   // per-pixel residual math in T (float64 is scarce on this GPU); the
   // thread's chi^2 partial of at most RY * 4 terms joins the block sum in
   // float64.  A row's inputs are all loaded before its first store.
@@ -455,7 +455,7 @@ int conv_variant_fast(int v) {
 }
 
 template <typename T, int BX, int BY, int RY, int NC>
-static void fwd_launch(const ConvWork* work, int n, const ImageDev* imgs, double* chi2_partial, void* const* model_out,
+static void fwd_launch(const ConvWork* work, int n, const ImageDev* imgs, double* chi2_partial, const ModelOut& model_out,
                        const int* skip, int trial, int store_sw, int* status, int kmax, cudaStream_t st) {
   if constexpr (NC == 0 || (sizeof(T) == 4 && fast_shape(BX, BY, RY)))
     forward_conv_kernel<T, BX, BY, RY, NC><<<n, BX * BY, corr_smem_bytes<T, BX, BY, RY>(kmax), st>>>(
@@ -489,7 +489,7 @@ static std::vector<ConvRange> launch_ranges(int v, const ConvRange* ranges, int 
 
 template <typename T>
 void launch_forward_conv(int v, const ConvWork* work, const ConvRange* ranges, int n_ranges, const ImageDev* imgs,
-                         double* chi2_partial, void* const* model_out, const int* skip, int trial, int store_sw,
+                         double* chi2_partial, const ModelOut& model_out, const int* skip, int trial, int store_sw,
                          int* status, int kmax, cudaStream_t st) {
   for (const ConvRange& r : launch_ranges(v, ranges, n_ranges)) {
     const int nc = r.nc;
@@ -554,50 +554,41 @@ __device__ __forceinline__ double gather_sum(const double* __restrict__ partial,
   return v;   // thread 0
 }
 
-constexpr int SUM_GROUP_THREADS = 256;
-__global__ void __launch_bounds__(SUM_GROUP_THREADS) sum_groups_kernel(
-    const double* __restrict__ partial, const int* __restrict__ ptr, const int* __restrict__ idx,
-    double* __restrict__ out, double scale, const int* __restrict__ skip, const double* __restrict__ keep) {
-  __shared__ double red[SUM_GROUP_THREADS / 32];
-  const int g = blockIdx.x;
-  if (skip && skip[g]) {   // the group's forward did not run: its value is kept
-    if (threadIdx.x == 0) out[g] = keep[g];
+// chi^2 of the groups (the first n_groups CTAs: scale 1; a group whose forward did
+// not run keeps its value) and the gradient's components (scale -2; half the
+// negative of it is J^T W r), either part may be empty: one launch for both.
+constexpr int GATHER_THREADS = 128;
+__global__ void __launch_bounds__(GATHER_THREADS) gather_kernel(GatherPlan g) {
+  __shared__ double red[GATHER_THREADS / 32];
+  const int b = blockIdx.x;
+  if (b < g.n_groups) {
+    if (g.skip && g.skip[b]) {
+      if (threadIdx.x == 0) g.chi2[b] = g.keep[b];
+      return;
+    }
+    const double s = gather_sum<GATHER_THREADS, int>(g.chi2_partial, g.grp_idx, g.grp_ptr[b], g.grp_ptr[b + 1], red);
+    if (threadIdx.x == 0) g.chi2[b] = s;
     return;
   }
-  const double s = gather_sum<SUM_GROUP_THREADS, int>(partial, idx, ptr[g], ptr[g + 1], red);
-  if (threadIdx.x == 0) out[g] = scale * s;
-}
-
-__global__ void __launch_bounds__(128) sum_contrib_kernel(const double* __restrict__ partial,
-                                                          const int64_t* __restrict__ ptr,
-                                                          const int64_t* __restrict__ idx, double* __restrict__ out,
-                                                          double scale, double* __restrict__ half) {
-  __shared__ double red[4];
-  const int g = blockIdx.x;
-  const double s = gather_sum<128, int64_t>(partial, idx, ptr[g], ptr[g + 1], red);
+  const int p = b - g.n_groups;
+  const double s =
+      gather_sum<GATHER_THREADS, int64_t>(g.grad_partial, g.par_idx, g.par_ptr[p], g.par_ptr[p + 1], red);
   if (threadIdx.x == 0) {
-    out[g] = scale * s;
-    if (half) half[g] = -0.5 * (scale * s);
+    g.grad[p] = -2.0 * s;
+    if (g.jtwr) g.jtwr[p] = s;
   }
 }
 
-void launch_sum_groups(const double* partial, const int* ptr, const int* idx, int n_out, double* out, double scale,
-                       const int* skip, const double* keep, cudaStream_t st) {
-  if (n_out > 0)
-    sum_groups_kernel<<<n_out, SUM_GROUP_THREADS, 0, st>>>(partial, ptr, idx, out, scale, skip, keep);
-}
-
-void launch_sum_contrib(const double* partial, const int64_t* ptr, const int64_t* idx, int n_out, double* out,
-                        double scale, double* half, cudaStream_t st) {
-  if (n_out > 0) sum_contrib_kernel<<<n_out, 128, 0, st>>>(partial, ptr, idx, out, scale, half);
+void launch_gather(const GatherPlan& g, cudaStream_t st) {
+  if (g.n_groups + g.n_params > 0) gather_kernel<<<g.n_groups + g.n_params, GATHER_THREADS, 0, st>>>(g);
 }
 
 template void configure_conv<float>(int, int*);
 template void configure_conv<double>(int, int*);
 template void launch_jcol<float>(int, const JcolWork*, const ConvRange*, int, const SourceDev*, const ImageDev*, const float*, float*, int, cudaStream_t);
 template void launch_jcol<double>(int, const JcolWork*, const ConvRange*, int, const SourceDev*, const ImageDev*, const double*, double*, int, cudaStream_t);
-template void launch_forward_conv<float>(int, const ConvWork*, const ConvRange*, int, const ImageDev*, double*, void* const*, const int*, int, int, int*, int, cudaStream_t);
-template void launch_forward_conv<double>(int, const ConvWork*, const ConvRange*, int, const ImageDev*, double*, void* const*, const int*, int, int, int*, int, cudaStream_t);
+template void launch_forward_conv<float>(int, const ConvWork*, const ConvRange*, int, const ImageDev*, double*, const ModelOut&, const int*, int, int, int*, int, cudaStream_t);
+template void launch_forward_conv<double>(int, const ConvWork*, const ConvRange*, int, const ImageDev*, double*, const ModelOut&, const int*, int, int, int*, int, cudaStream_t);
 template void launch_adjoint_conv<float>(int, const ConvWork*, const ConvRange*, int, const ImageDev*, int, cudaStream_t);
 template void launch_adjoint_conv<double>(int, const ConvWork*, const ConvRange*, int, const ImageDev*, int, cudaStream_t);
 

@@ -243,11 +243,20 @@ struct ConvRange {
 };
 int conv_nc_of(int K4, int is_double);
 
+// where the model images go: up to MODEL_OUT_MAX pointers by value (the launch
+// copies them), else a device table; none: no model wanted
+constexpr int MODEL_OUT_MAX = 16;
+struct ModelOut {
+  int n = 0;
+  void* p[MODEL_OUT_MAX] = {};
+  void* const* table = nullptr;
+};
+
 // forward correlation of the galaxy layer with the flipped PSF + model
 // assembly + residual + chi^2 partials (and the model into model_out)
 template <typename T>
 void launch_forward_conv(int tile_variant, const ConvWork* work, const ConvRange* ranges, int n_ranges,
-                         const ImageDev* imgs, double* chi2_partial, void* const* model_out, const int* skip,
+                         const ImageDev* imgs, double* chi2_partial, const ModelOut& model_out, const int* skip,
                          int trial, int store_sw, int* status, int kmax, cudaStream_t st);
 
 // adjoint correlation: adj = P (correlate) w r over the galaxy layer
@@ -272,11 +281,21 @@ int conv_tile_h(int variant);
 int conv_threads(int variant);
 constexpr int N_CONV_VARIANTS = 7;
 
-void launch_sum_groups(const double* partial, const int* ptr, const int* idx, int n_out, double* out,
-                       double scale, const int* skip, const double* keep, cudaStream_t st);
-// out = scale * sum; half (nullable): -sum * scale / 2, the J^T W r of a gradient
-void launch_sum_contrib(const double* partial, const int64_t* ptr, const int64_t* idx, int n_out, double* out,
-                        double scale, double* half, cudaStream_t st);
+// the float64 gathers of an evaluation: chi^2 per group from the correlation tiles'
+// partials, the gradient (and J^T W r) from the render tiles'
+struct GatherPlan {
+  const double* chi2_partial;
+  const int *grp_ptr, *grp_idx;
+  int n_groups;            // 0: no chi^2
+  double* chi2;
+  const int* skip;         // groups whose chi^2 is keep[g]
+  const double* keep;
+  const double* grad_partial;
+  const int64_t *par_ptr, *par_idx;
+  int n_params;            // 0: no gradient
+  double *grad, *jtwr;     // jtwr nullable
+};
+void launch_gather(const GatherPlan& g, cudaStream_t st);
 
 // J^T W J in two passes (see ap_gram.cu).  A source pair is two sources
 // (A <= B) reaching a common image tile; its block holds the m_A x m_B
