@@ -302,6 +302,11 @@ __global__ void __launch_bounds__(FftShape<N>::NT) psf_spectrum_kernel(const flo
   }
 }
 
+// asynchronous 4-byte copy global -> shared, zero where !in
+__device__ __forceinline__ void copy_async4(unsigned dst, const float* src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+
 template <int N>
 __global__ void __launch_bounds__(FftShape<N>::NTR, FftShape<N>::MINB) jcol_fft_kernel(const JcolFftWork* __restrict__ work,
                                                                    const SourceDev* __restrict__ srcs,
@@ -318,22 +323,32 @@ __global__ void __launch_bounds__(FftShape<N>::NTR, FftShape<N>::MINB) jcol_fft_
   const ImageDev& im = imgs[sd.image];
   const int h = im.h, K = im.K, B = N - K + 1;
   const int bh = sd.box[1] - sd.box[0], bw = sd.box[3] - sd.box[2];
-  const float* d1 = dbuf + sd.d_off + w.k * (int64_t)bh * bw;
   for (int i = threadIdx.x; i < N; i += NT) tw[i] = tw_g[i];
+  const float2* S = reinterpret_cast<const float2*>(N == 64 ? im.spec64 : im.spec128);
+  constexpr int RSTEP = NT / N;   // rows per sweep (the threads past RSTEP * N idle)
+  const int col_j = threadIdx.x % N, row_j = threadIdx.x / N;
   // rows: view A row r = block rows 2r (real part) and 2r + 1 (imaginary
   // part) of the derivative image on the block grown by K - 1, zero outside
-  // the box; loaded with consecutive threads on consecutive pixels of a row
-  // (coalesced), then transformed in place
-  const int y0 = w.by0 - h, x0 = w.bx0 - h;
-#pragma unroll 4
-  for (int idx = threadIdx.x; idx < H * N; idx += NT) {
-    const int r = idx / N, v = idx % N;
-    const int y = y0 + 2 * r, x = x0 + v;
+  // the box; asynchronous copies with consecutive threads on consecutive pixels
+  // of a row, all in flight together (through registers a block waited for every
+  // group of four; with the two prefetches below, 40 small cutouts: 270 -> 240 us,
+  // a 1024^2 field 157 -> 154, four joint 1024^2 exposures 1391 -> 1376), then transformed in place
+  if (row_j < RSTEP) {
+    const int x = w.bx0 - h + col_j, y0 = w.by0 - h;
     const bool inx = x >= 0 && x < bw;
-    const float a = (inx && y >= 0 && y < bh) ? d1[(int64_t)y * bw + x] : 0.f;
-    const float b = (inx && y + 1 >= 0 && y + 1 < bh) ? d1[(int64_t)(y + 1) * bw + x] : 0.f;
-    sm[r * LDA + v] = make_float2(a, b);
+    const float* src = dbuf + sd.d_off + w.k * (int64_t)bh * bw + (inx ? x : 0);
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(sm + col_j);
+#pragma unroll 8
+    for (int r = row_j; r < N; r += RSTEP) {
+      const int y = y0 + r;
+      const bool in = inx && y >= 0 && y < bh;
+      copy_async4(dst + ((r >> 1) * LDA * 8 + (r & 1) * 4), src + (in ? (int64_t)y * bw : 0), in);
+    }
   }
+  // meanwhile the PSF spectrum (columns 0..N/2 of its N rows) on its way into the L1
+  for (int i = threadIdx.x; i < N * (H / 16 + 1); i += NT)
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(S + (i / (H / 16 + 1)) * N + (i % (H / 16 + 1)) * 16));
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   auto ld_rows = [&](int r, int v) { return sm[r * LDA + v]; };
   auto st_a = [&](int r, int k, float2 z) { sm[r * LDA + k] = z; };
@@ -354,10 +369,15 @@ __global__ void __launch_bounds__(FftShape<N>::NTR, FftShape<N>::MINB) jcol_fft_
     }
     return make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y + zm.y));
   };
-  const float2* S = reinterpret_cast<const float2*>(N == 64 ? im.spec64 : im.spec128);
   auto mul = [&](int k, int n, float2 z) { return c_mul(z, __ldg(S + n * N + k)); };
   fft_lines_product<N, NT, LDB, 1>(sm, H + 1, tw, ld_split, mul);
   __syncthreads();
+  // the outputs' weights on their way into the L1 during the last pass
+  for (int i = threadIdx.x; i < B * (N / 32); i += NT) {
+    const int oi = sd.box[0] + w.by0 + i / (N / 32), oc = sd.box[2] + w.bx0 + (i % (N / 32)) * 32;
+    if (oi >= sd.sup[0] && oi < sd.sup[1] && oc >= sd.sup[2] && oc < sd.sup[3])
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(im.sw + (int64_t)oi * im.W + oc));
+  }
   // inverse rows: the first stage packs the row pairs again, W = Y_a + i Y_b
   // over the full row (Hermitian extension of the half spectra); the
   // inverse of W is row a + i row b
@@ -376,10 +396,9 @@ __global__ void __launch_bounds__(FftShape<N>::NTR, FftShape<N>::MINB) jcol_fft_
   // outputs: block rows / columns [0, B) sit at [K - 1, N) of the circular
   // result; thread t takes column t mod N of rows t / N, t / N + NT / N, ...,
   // stored sqrt(w)-scaled into the source's column blocks
-  constexpr int RSTEP = NT / N;   // rows per sweep (the threads past RSTEP * N idle)
-  const int j = threadIdx.x % N;
+  const int j = col_j;
   const int oj = sd.box[2] + w.bx0 + j;
-  if (threadIdx.x < RSTEP * N && j < B && oj >= sd.sup[2] && oj < sd.sup[3]) {
+  if (row_j < RSTEP && j < B && oj >= sd.sup[2] && oj < sd.sup[3]) {
     // the thread's column of the blocks: the tile column is fixed, a row adds
     // a tile row's stride per 16 rows and a line of the tile per row
     const int64_t tile_row = (int64_t)sd.gt[2] * sd.nfree * TILE_THREADS;
@@ -389,7 +408,7 @@ __global__ void __launch_bounds__(FftShape<N>::NTR, FftShape<N>::MINB) jcol_fft_
     const float* z = reinterpret_cast<const float*>(sm + (j + K - 1));
     constexpr int RUN = 8;   // rows whose weights are loaded together
 #pragma unroll 1
-    for (int i = i0 + threadIdx.x / N; i < i1; i += RUN * RSTEP) {
+    for (int i = i0 + row_j; i < i1; i += RUN * RSTEP) {
       float sv[RUN];
 #pragma unroll
       for (int u = 0; u < RUN; ++u) sv[u] = i + u * RSTEP < i1 ? __ldg(sw + (int64_t)(r0 + i + u * RSTEP) * im.W) : 0.f;
