@@ -116,6 +116,49 @@ __device__ __forceinline__ float p_rcp(float x) {
 }
 __device__ __forceinline__ double p_rcp(double x) { return 1.0 / x; }
 
+// A thread's two pixels in one packed float32 value: products, sums and fmas of
+// both are one instruction (with the roundings of two), the special functions
+// two.  The value render's profile code takes V = F2, float or double.  Its launch
+// on a field of 281 galaxies and 703 stars (1536^2): 81 -> 72 us, on twelve joint
+// 2048^2 exposures 1066 -> 948 us.  (The derivative render is not packed: 16 sums a
+// thread instead of 8 at a time cost it a third of its warps, 4.83 -> 4.99 ms.)
+struct F2 {
+  float2 v;
+};
+template <typename V, typename T>
+__device__ __forceinline__ V p_all(T x) {
+  if constexpr (sizeof(V) == 2 * sizeof(T)) return F2{make_float2(x, x)};
+  else return x;
+}
+#define AP_F2_BITS(a) reinterpret_cast<const unsigned long long&>((a).v)
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(reinterpret_cast<unsigned long long&>(r.v)) : "l"(AP_F2_BITS(a)), "l"(AP_F2_BITS(b)));
+  return r;
+}
+__device__ __forceinline__ F2 operator*(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(reinterpret_cast<unsigned long long&>(r.v)) : "l"(AP_F2_BITS(a)), "l"(AP_F2_BITS(b)));
+  return r;
+}
+__device__ __forceinline__ F2 p_fma(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(reinterpret_cast<unsigned long long&>(r.v))
+      : "l"(AP_F2_BITS(a)), "l"(AP_F2_BITS(b)), "l"(AP_F2_BITS(c)));
+  return r;
+}
+#undef AP_F2_BITS
+__device__ __forceinline__ float p_fma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double p_fma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ F2 p_exp2(F2 a) { return F2{make_float2(p_exp2(a.v.x), p_exp2(a.v.y))}; }
+__device__ __forceinline__ F2 p_log2(F2 a) { return F2{make_float2(p_log2(a.v.x), p_log2(a.v.y))}; }
+
+// sources without a radial profile: the skies, a PSF star and a live PSF
+__device__ __forceinline__ bool no_profile(int type) {
+  return type == AP_SKY_FLAT || type == AP_SKY_PLANE || type == AP_PSF_STAR || type == AP_LIVE_PSF_SRC;
+}
+
 constexpr double LOG2E = 1.4426950408889634074;
 constexpr double LN2 = 0.69314718055994530942;
 
@@ -422,7 +465,7 @@ __device__ __forceinline__ void psf_bilinear(const T* __restrict__ map, int K, i
 // value of one source on one pixel: amp * sum_ab (w_a/2)(w_b/2) f(node_ab)
 // ---------------------------------------------------------------------------
 template <typename T, int Q>
-__device__ __forceinline__ T pixel_value(int type, const SrcPar<T>& P, int i, int j, const ImageDev& im) {
+__device__ __forceinline__ T other_value(int type, const SrcPar<T>& P, int i, int j, const ImageDev& im) {
   if (type == AP_LIVE_PSF_SRC) return (T)0;   // a live PSF draws nothing itself
   if (type == AP_SKY_FLAT) return P.area * P.k0;
   if (type == AP_PSF_STAR) {
@@ -445,52 +488,91 @@ __device__ __forceinline__ T pixel_value(int type, const SrcPar<T>& P, int i, in
     }
     return P.k0 * acc;
   }
-  if (type == AP_SKY_PLANE) {
-    T du = (T)j + (T)0.5 - P.fx;
-    T dv = (T)i + (T)0.5 - P.fy;
-    T dxw = P.m00 * du + P.m01 * dv;
-    T dyw = P.m10 * du + P.m11 * dv;
-    return P.area * (P.k0 + P.k1 * dxw + P.k2 * dyw);
-  }
-  const T du0 = (T)(j - P.jc) + ((T)0.5 - P.fx);
-  const T dv0 = (T)(i - P.ic) + ((T)0.5 - P.fy);
-  const T x0 = P.m00 * du0 + P.m01 * dv0;
-  const T y0 = P.m10 * du0 + P.m11 * dv0;
-  T acc = (T)0;
-  // Per Sersic node 7 float32 instructions and three special-function ones
-  // (lg2 at half the rate of ex2), which bound the loop.
+  T du = (T)j + (T)0.5 - P.fx;
+  T dv = (T)i + (T)0.5 - P.fy;
+  T dxw = P.m00 * du + P.m01 * dv;
+  T dyw = P.m10 * du + P.m11 * dv;
+  return P.area * (P.k0 + P.k1 * dxw + P.k2 * dyw);
+}
+
+// (dv0 the pixels' row coordinates, du0 the column's)
+template <typename V, typename T, int Q>
+__device__ __forceinline__ V profile_value(int type, const SrcPar<T>& P, T du0, V dv0) {
+  auto B = [](T x) { return p_all<V, T>(x); };
+  const V x0 = p_fma(B(P.m01), dv0, B(P.m00 * du0));
+  const V y0 = p_fma(B(P.m11), dv0, B(P.m10 * du0));
+  V acc = B((T)0);
+  // Per Sersic node 7 float32 instructions (packed, for two pixels) and three
+  // special-function ones a pixel (lg2 at half the rate of ex2), which bound the
+  // loop.
 #pragma unroll
   for (int b = 0; b < Q; ++b) {
     const T hb = gl_hu<T>(Q, b);
-    const T xb = x0 + P.m01 * hb, yb = y0 + P.m11 * hb;
-    T accb = (T)0;
+    const V xb = x0 + B(P.m01 * hb), yb = y0 + B(P.m11 * hb);
+    V accb = B((T)0);
     if (type == AP_SERSIC || type == AP_EXPONENTIAL) {
 #pragma unroll
       for (int a = 0; a < Q; ++a) {
         const T ha = gl_hu<T>(Q, a);
-        const T x = xb + P.m00 * ha, y = yb + P.m10 * ha;
-        const T u = fma(x, x, fma(y, y, P.k1));
-        const T t = p_exp2(P.k0 * p_log2(u));                 // (R/Re)^(1/n)
-        accb += gl_hw<T>(Q, a) * p_exp2(fma(-P.k2, t, P.k2));
+        const V x = xb + B(P.m00 * ha), y = yb + B(P.m10 * ha);
+        const V u = p_fma(x, x, p_fma(y, y, B(P.k1)));
+        const V t = p_exp2(B(P.k0) * p_log2(u));              // (R/Re)^(1/n)
+        accb = p_fma(B(gl_hw<T>(Q, a)), p_exp2(p_fma(B(-P.k2), t, B(P.k2))), accb);
       }
     } else if (type == AP_GAUSSIAN) {
 #pragma unroll
       for (int a = 0; a < Q; ++a) {
         const T ha = gl_hu<T>(Q, a);
-        const T x = xb + P.m00 * ha, y = yb + P.m10 * ha;
-        accb += gl_hw<T>(Q, a) * p_exp2(P.k0 * fma(x, x, y * y));
+        const V x = xb + B(P.m00 * ha), y = yb + B(P.m10 * ha);
+        accb = p_fma(B(gl_hw<T>(Q, a)), p_exp2(B(P.k0) * p_fma(x, x, y * y)), accb);
       }
     } else {  // Moffat: (1 + rho^2/Rd^2)^-n
 #pragma unroll
       for (int a = 0; a < Q; ++a) {
         const T ha = gl_hu<T>(Q, a);
-        const T x = xb + P.m00 * ha, y = yb + P.m10 * ha;
-        accb += gl_hw<T>(Q, a) * p_exp2(-P.k2 * p_log2(fma(x, x, fma(y, y, (T)1))));
+        const V x = xb + B(P.m00 * ha), y = yb + B(P.m10 * ha);
+        accb = p_fma(B(gl_hw<T>(Q, a)), p_exp2(B(-P.k2) * p_log2(p_fma(x, x, p_fma(y, y, B((T)1))))), accb);
       }
     }
-    acc += gl_hw<T>(Q, b) * accb;
+    acc = p_fma(B(gl_hw<T>(Q, b)), accb, acc);
   }
-  return P.amp * acc;
+  return B(P.amp) * acc;
+}
+
+template <typename T>
+__device__ __forceinline__ T row_coord(const SrcPar<T>& P, int i) {
+  return (T)(i - P.ic) + ((T)0.5 - P.fy);
+}
+template <typename T>
+__device__ __forceinline__ T col_coord(const SrcPar<T>& P, int j) {
+  return (T)(j - P.jc) + ((T)0.5 - P.fx);
+}
+
+template <typename T, int Q>
+__device__ __forceinline__ T pixel_value(int type, const SrcPar<T>& P, int i, int j, const ImageDev& im) {
+  if (no_profile(type)) return other_value<T, Q>(type, P, i, j, im);
+  return profile_value<T, T, Q>(type, P, col_coord(P, j), row_coord(P, i));
+}
+
+// a thread's two pixels, rows i0 and i1 of column j
+template <int Q>
+__device__ __forceinline__ void pair_value(int type, const SrcPar<float>& P, int i0, int i1, int j, const ImageDev& im,
+                                           float& v0, float& v1) {
+  if (no_profile(type)) {
+    v0 = other_value<float, Q>(type, P, i0, j, im);
+    v1 = other_value<float, Q>(type, P, i1, j, im);
+    return;
+  }
+  const F2 v = profile_value<F2, float, Q>(type, P, col_coord(P, j),
+                                           F2{make_float2(row_coord(P, i0), row_coord(P, i1))});
+  v0 = v.v.x;
+  v1 = v.v.y;
+}
+template <int Q>
+__device__ __forceinline__ void pair_value(int type, const SrcPar<double>& P, int i0, int i1, int j, const ImageDev& im,
+                                           double& v0, double& v1) {
+  v0 = pixel_value<double, Q>(type, P, i0, j, im);
+  v1 = pixel_value<double, Q>(type, P, i1, j, im);
 }
 
 // ---------------------------------------------------------------------------
@@ -527,8 +609,8 @@ __global__ void __launch_bounds__(RENDER_THREADS) render_kernel(const TileWork* 
     const bool in1 = cin && i1 >= sd.box[0] && i1 < sd.box[1];
     if (in0 || in1) {
       const SrcPar<T> P = par[s];
-      const T v0 = pixel_value<T, Q>(sd.type, P, i0, j, im);
-      const T v1 = pixel_value<T, Q>(sd.type, P, i1, j, im);
+      T v0, v1;
+      pair_value<Q>(sd.type, P, i0, i1, j, im, v0, v1);
       acc0 += in0 ? v0 : (T)0;
       acc1 += in1 ? v1 : (T)0;
     }
