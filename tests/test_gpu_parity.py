@@ -779,3 +779,53 @@ def test_sersic_bn_table(n):
     np.testing.assert_allclose(_np(c), O.chi2(pr, theta), rtol=TOL_F64, atol=0)
     assert_grad_close(_np(g), O.gradient(pr, theta), grad_scale(pr, theta), 1e-8)
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("ns,nm", [(0, 0), (1, 2), (2, 0), (2, 5), (3, 3), (6, 6), (1, 18), (2, 16), (3, 24), (4, 22),
+                                   (5, 30), (6, 28)])
+def test_jtwj_and_solve_at_column_count_edges(ns, nm):
+    """One 16 x 16 tile with 3, 16, 17, 32, 33, 63, 64, 65, 96, 97, 128 and 129
+    free columns (the edges of the tile Gram's 16-column forms, of its 64-column
+    off-diagonal blocks and of the dense solve): J^T W J against the oracle to the
+    tolerance of the other comparisons, the step against the device's own damped
+    matrix (kappa at most 2 n at lambda = 1, so 1e-8 is far above rounding)."""
+    pr = with_data(configs.crowded_field(f"edge_{ns}_{nm}", configs.SEED_BASE + 90 + ns, 16, 16, ns, nm,
+                                         configs.psf_moffat(5, 2.5)))
+    assert pr.n_params == 7 * ns + 3 * nm + 3
+    ctx = device_context(pr, "mixed")
+    ref, _ = O.normal_equations(pr, pr.theta_init)
+    jtwr, csr = ctx.normal_eq(pr.theta_init)
+    JtWJ = ctx.jtwj_dense(csr)
+    d = np.sqrt(np.maximum(np.diag(ref), 1e-300))
+    assert (np.abs(JtWJ - ref) / np.outer(d, d)).max() <= TOL_GRAD
+    delta, _ = ctx.lm_solve(np.array([1.0]))
+    assert_step_close(_np(delta), np.linalg.solve(damped_matrix(JtWJ, 1.0), _np(jtwr)), JtWJ, 1.0, 1e-8)
+    assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("n", [16, 17])
+def test_model_images_past_the_argument_pointers(n):
+    """Up to 16 model images travel as kernel arguments, more as a device table."""
+    pr = problem("mixed", seed=configs.SEED_BASE + 27, H=20, W=23, K=5, n_images=n)
+    got = device_context(pr, "mixed").render(pr.theta_init)
+    for a, b in zip(got, O.model_images(pr, pr.theta_init)):
+        assert np.abs(_np(a) - b).max() <= TOL_MODEL * np.abs(b).max()
+
+
+def test_replayed_evaluation_between_lm_calls():
+    """An evaluation captured in a graph and replayed between LM calls: the
+    continued fit evaluates at its theta again, as after a direct call."""
+    pr = get_case("mixed_rot")
+    ctx, a, _, _ = _lm_paths(pr, 1e-3, 4, "f64")
+    theta = torch.as_tensor(pr.theta_true, dtype=torch.float64, device="cuda")
+    ctx.eval(theta)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chi2, _ = ctx.eval(theta)
+    ctx.lm_iterate(pr.theta_init, np.full(pr.n_groups, 1e-3), 2)
+    graph.replay()
+    th, _, c, log = ctx.lm_continue(2, log=True)
+    np.testing.assert_allclose(_np(chi2), O.chi2(pr, pr.theta_true), rtol=TOL_F64, atol=0)
+    np.testing.assert_array_equal(log[:, :, 3], a[2][2:, :, 3])
+    np.testing.assert_allclose(_np(c), a[1], rtol=1e-12)
+    np.testing.assert_allclose(_np(th), a[0], rtol=1e-10, atol=1e-12)
