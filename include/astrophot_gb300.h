@@ -86,11 +86,8 @@ typedef struct {
                         autotuned; v >= 1 forces variant v - 1 of
                         ap_get_conv_variant() (AP_ERR_ARG from ap_set_problem
                         if it does not fit the problem's largest PSF)         */
-  int gram_tc_min;   /* mixed form, J^T W J tile Grams: 0 = chosen by timing in
-                        ap_set_problem; k >= 1: tiles with k .. 128 Jacobian
-                        columns run on the tensor-core (tcgen05) kernel, the
-                        others on the warp-MMA kernel (k > 128: none); k is
-                        rounded up to 1 + a multiple of 16                     */
+  int gram_tc_min;   /* accepted (>= 0) and without effect: the J^T W J tile
+                        Grams run in one form                                 */
 } ap_options;
 
 /* Jacobian-column convolution modes.  AUTO times both on the problem in

@@ -33,8 +33,9 @@
 // halves of the operands -- no less than the warp MMAs; as built before (producer
 // warps gathering columns and storing swizzled heads and tails) it took 21 700
 // clocks per tile.  J^T W J of the 12 x 2048^2 joint fit (196 608 tiles, 38
-// columns on average) 14.2 -> 5.5 ms, of the 1536^2 crowded field 1.43 -> 0.65 ms,
-// of 64 cutouts 230 -> 80 us.
+// columns on average) 14.2 -> 6.1 ms, of the 1536^2 crowded field 1.43 -> 0.71 ms,
+// of 64 cutouts 230 -> 84 us (5.5, 0.65 and 80 before each MMA step was summed
+// outside the accumulator).
 //
 // Float64 path: one CTA per tile, columns gathered into shared memory, products
 // on the CUDA cores, float64 blocks.
