@@ -480,10 +480,11 @@ bool capturing(cudaStream_t st) {
 
 // Nothing to clear if no LM iteration has run since the last time.  A captured
 // call always clears, as its graph may be replayed after an iteration, and so does
-// every call once iterations have been captured.
+// every call once iterations have been captured.  Its clearing is only recorded:
+// the flags on the device stay as they are, and the next direct call clears them.
 int drop_lm_reuse(ap_ctx* c, cudaStream_t st) {
   if (!c->fwd_flags_set && !c->fwd_flags_captured && !capturing(st)) return AP_OK;
-  c->fwd_flags_set = false;
+  if (!capturing(st)) c->fwd_flags_set = false;
   CUDA_TRY(c, cudaMemsetAsync(c->d_fwd_valid, 0, (size_t)std::max(c->n_groups, 1) * sizeof(int), st));
   return AP_OK;
 }
