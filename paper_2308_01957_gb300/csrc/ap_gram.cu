@@ -509,14 +509,20 @@ template <> struct TileSum<float2> {
     lo = __fadd_rn(lo, v.y);
   }
   __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
+  __device__ __forceinline__ bool in_range() const { return isfinite(hi); }   // (an infinite or NaN hi stays one)
 };
 template <> struct TileSum<double> {
   double s = 0.0;
   __device__ __forceinline__ void add(double v) { s += v; }
   __device__ __forceinline__ double get() const { return s; }
+  __device__ __forceinline__ bool in_range() const { return true; }
 };
+__device__ __forceinline__ double as_double(float2 v) { return (double)v.x + (double)v.y; }
+__device__ __forceinline__ double as_double(double v) { return v; }
 
-// entry values src[k ne], k = k0, k0 + step, ... below cnt: eight loads in flight
+// entry values src[k ne], k = k0, k0 + step, ... below cnt: eight loads in flight.
+// A float sum that leaves float32's range (tile entries up to 3.4e38 each) is
+// taken again in float64, which holds it (a comparison per sum: J^T W J within 0.5 %).
 template <typename V>
 __device__ __forceinline__ double tile_sum(const V* __restrict__ src, int ne, int k0, int step, int cnt) {
   TileSum<V> acc;
@@ -535,7 +541,11 @@ __device__ __forceinline__ double tile_sum(const V* __restrict__ src, int ne, in
 #pragma unroll
   for (int u = 0; u < 7; ++u)
     if (k + u * step < cnt) acc.add(v[u]);
-  return acc.get();
+  if (acc.in_range()) return acc.get();
+  double s = 0.0;
+#pragma unroll 1
+  for (k = k0; k < cnt; k += step) s += as_double(src[(int64_t)k * ne]);
+  return s;
 }
 
 __device__ __forceinline__ void gram_write(const GramPair& gp, const int64_t* __restrict__ pos, int e, double s,
