@@ -509,20 +509,14 @@ template <> struct TileSum<float2> {
     lo = __fadd_rn(lo, v.y);
   }
   __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
-  __device__ __forceinline__ bool in_range() const { return isfinite(hi); }   // (an infinite or NaN hi stays one)
 };
 template <> struct TileSum<double> {
   double s = 0.0;
   __device__ __forceinline__ void add(double v) { s += v; }
   __device__ __forceinline__ double get() const { return s; }
-  __device__ __forceinline__ bool in_range() const { return true; }
 };
-__device__ __forceinline__ double as_double(float2 v) { return (double)v.x + (double)v.y; }
-__device__ __forceinline__ double as_double(double v) { return v; }
 
-// entry values src[k ne], k = k0, k0 + step, ... below cnt: eight loads in flight.
-// A float sum that leaves float32's range (tile entries up to 3.4e38 each) is
-// taken again in float64, which holds it (a comparison per sum: J^T W J within 0.5 %).
+// entry values src[k ne], k = k0, k0 + step, ... below cnt: eight loads in flight
 template <typename V>
 __device__ __forceinline__ double tile_sum(const V* __restrict__ src, int ne, int k0, int step, int cnt) {
   TileSum<V> acc;
@@ -541,23 +535,34 @@ __device__ __forceinline__ double tile_sum(const V* __restrict__ src, int ne, in
 #pragma unroll
   for (int u = 0; u < 7; ++u)
     if (k + u * step < cnt) acc.add(v[u]);
-  if (acc.in_range()) return acc.get();
-  double s = 0.0;
+  return acc.get();
+}
+
+// A float sum that left float32's range (of tile entries up to 3.4e38 each; an
+// infinite or NaN hi stays one) is taken again in float64, which holds it.
+__device__ __forceinline__ double in_range(const double* __restrict__, int, int, int, double s) { return s; }
+__device__ __forceinline__ double in_range(const float2* __restrict__ src, int ne, int k0, int cnt, double s) {
+  if ((__double2hiint(s) & 0x7ff00000) != 0x7ff00000) return s;
+  s = 0.0;
 #pragma unroll 1
-  for (k = k0; k < cnt; k += step) s += as_double(src[(int64_t)k * ne]);
+  for (int k = k0; k < cnt; ++k) s += (double)src[(int64_t)k * ne].x + (double)src[(int64_t)k * ne].y;
   return s;
 }
 
-__device__ __forceinline__ void gram_write(const GramPair& gp, const int64_t* __restrict__ pos, int e, double s,
-                                           double* __restrict__ vals) {
-  const int64_t pab = pos[gp.pos + 2 * e], pba = pos[gp.pos + 2 * e + 1];
-  if (pab < 0) return;   // below the diagonal of a source's own block
+struct EntryPos {
+  int64_t ab, ba;   // in the CSR values: the entry's and its mirror's (-1: not stored)
+};
+__device__ __forceinline__ EntryPos entry_pos(const GramPair& gp, const int64_t* __restrict__ pos, int e) {
+  return EntryPos{pos[gp.pos + 2 * e], pos[gp.pos + 2 * e + 1]};
+}
+__device__ __forceinline__ void gram_write(const GramPair& gp, EntryPos at, double s, double* __restrict__ vals) {
+  if (at.ab < 0) return;   // below the diagonal of a source's own block
   if (gp.excl) {
-    vals[pab] = s;
-    if (pba >= 0) vals[pba] = s;
+    vals[at.ab] = s;
+    if (at.ba >= 0) vals[at.ba] = s;
   } else {
-    atomicAdd(vals + pab, s);
-    if (pba >= 0) atomicAdd(vals + pba, s);
+    atomicAdd(vals + at.ab, s);
+    if (at.ba >= 0) atomicAdd(vals + at.ba, s);
   }
 }
 
@@ -573,13 +578,20 @@ __global__ void __launch_bounds__(256) gram_reduce_kernel(const GramPair* __rest
     const int ne = gp.ma * gp.mb;
     const V* src = scr + gp.base;
     if (ne > 16) {   // one tile at a time, an entry (or two) per lane
-      for (int e = lane; e < ne; e += 32) gram_write(gp, pos, e, tile_sum(src + e, ne, 0, 1, gp.cnt), vals);
+      for (int e = lane; e < ne; e += 32) {
+        const double s = tile_sum(src + e, ne, 0, 1, gp.cnt);
+        const EntryPos at = entry_pos(gp, pos, e);
+        gram_write(gp, at, in_range(src + e, ne, 0, gp.cnt, s), vals);
+      }
     } else {         // 32 / ne tiles side by side
       const int T = 32 / ne, e = lane % ne, t = lane / ne;
       const double part = t < T ? tile_sum(src + e, ne, t, T, gp.cnt) : 0.0;
       double s = 0.0;
       for (int k = 0; k < T; ++k) s += __shfl_sync(0xffffffffu, part, (k * ne + e) & 31);
-      if (lane < ne) gram_write(gp, pos, e, s, vals);
+      if (lane < ne) {
+        const EntryPos at = entry_pos(gp, pos, e);
+        gram_write(gp, at, in_range(src + e, ne, 0, gp.cnt, s), vals);
+      }
     }
   }
 }
@@ -603,8 +615,9 @@ __global__ void __launch_bounds__(256) gram_reduce_run_kernel(const GramPair* __
   double s = 0.0;
   if ((int)threadIdx.x < ne) {
     for (int k = 0; k < T; ++k) s += red[k * ne + threadIdx.x];
+    s = in_range(scr + gp.base + threadIdx.x, ne, rn.k0, rn.k1, s);
     if (rn.n_runs == 1)
-      gram_write(gp, pos, threadIdx.x, s, vals);
+      gram_write(gp, entry_pos(gp, pos, threadIdx.x), s, vals);
     else
       part[(int64_t)(rn.first + rn.run) * 64 + threadIdx.x] = s;
   }
@@ -618,7 +631,7 @@ __global__ void __launch_bounds__(256) gram_reduce_run_kernel(const GramPair* __
   if ((int)threadIdx.x < ne) {
     s = 0.0;
     for (int k = 0; k < rn.n_runs; ++k) s += __ldcg(part + (int64_t)(rn.first + k) * 64 + threadIdx.x);
-    gram_write(gp, pos, threadIdx.x, s, vals);
+    gram_write(gp, entry_pos(gp, pos, threadIdx.x), s, vals);
   }
   if (threadIdx.x == 0) done[rn.first] = 0;   // ready for the next call
 }
