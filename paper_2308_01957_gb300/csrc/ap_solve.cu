@@ -11,6 +11,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <cfloat>
 
 #include "ap_internal.cuh"
 
@@ -98,16 +99,8 @@ __global__ void __launch_bounds__(CHOL_THREADS) chol_kernel(
   double* A = sm;                                        // rows 0..n - 1, and the right-hand side as row n
   double* D = A + (max_n + 1) * chol_pitch(max_n);       // damping diagonal
   double* z = D + max_n;                                 // D^-1 L^-1 b
-  double* inv = z + max_n;                               // reciprocal pivots, 0 where the pivot fails
+  double* inv = z + max_n;                               // reciprocal pivots
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // hardware seed (20 bits) and two Newton steps, r <- r + r (1 - d r)
-  auto reciprocal = [](double d) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    r = fma(r, fma(-d, r, 1.0), r);
-    r = fma(r, fma(-d, r, 1.0), r);
-    return d > 0.0 && isfinite(d) && isfinite(r) ? r : 0.0;
-  };
   double d0 = 0.0;
   if (tid < n) {
     const int64_t e = dpos[gp[tid]];
@@ -131,18 +124,21 @@ __global__ void __launch_bounds__(CHOL_THREADS) chol_kernel(
     }
     __syncthreads();
     if (tid < n) A[tid * P + tid] += lam * D[tid];
-    if (tid == 0 && n > 0) inv[0] = reciprocal(A[0]);
+    if (tid == 0 && n > 0) inv[0] = 1.0 / A[0];
     __syncthreads();
     ok = true;
     for (int k = 0; k < n; ++k) {
-      const double iv = inv[k];
-      if (iv == 0.0) {   // the same for every thread
+      const double d = A[k * P + k], iv = inv[k];
+      // 2^-1022 <= d < 2^1022 (one integer comparison, the same for every thread):
+      // 1 / d is a normal number; other positive pivots divide
+      const bool normal = (unsigned)(__double2hiint(d) - 0x00100000) < 0x7fd00000u - 0x00100000u;
+      if (!normal && (!(d > 0.0) || !isfinite(d))) {
         ok = false;
         break;
       }
       const int r = k + 1 + (tid & 63), q = tid >> 6;
       if (r <= n) {
-        const double l = A[r * P + k] * iv;
+        const double l = normal ? A[r * P + k] * iv : A[r * P + k] / d;
         double* row = A + r * P;
         const int c1 = r < n ? r : n - 1;
 #pragma unroll 4
@@ -151,7 +147,7 @@ __global__ void __launch_bounds__(CHOL_THREADS) chol_kernel(
           if (r < n) A[k * P + r] = l;
           else z[k] = l;
         }
-        if (tid == 0 && r < n) inv[r] = reciprocal(row[r]);
+        if (tid == 0 && r < n) inv[r] = 1.0 / row[r];
       }
       __syncthreads();
     }
