@@ -92,8 +92,9 @@ struct SrcPar {
                          // the image centre in pixels (W/2, H/2)
   T area;
   T amp;                 // value scale: area Ie, area F norm
-  T k0, k1, k2;          // Sersic: 1/(2n), softening of u, b log2(e); Gaussian: -log2(e)/2;
-                         // Moffat: n; sky: the slot values; PSF star: F, map centre
+  T k0, k1, k2;          // Sersic: 1/(2n), softening of u, b log2(e); Gaussian: -log2(e)/2,
+                         // weight of the derivative sums; Moffat: -, weight, n; sky: the slot values;
+                         // PSF star: F, map centre
   // derivative coefficients: D0 = c0x Sx + c0y Sy, D1 = c1x Sx + c1y Sy,
   // D2 = c2 Syy + c2s S1, D3 = c3 Sxy, then c4a, c4b, c5a, c5b, c6 by type
   T c0x, c0y, c1x, c1y, c2, c2s, c3, c4a, c4b, c5a, c5b, c6;

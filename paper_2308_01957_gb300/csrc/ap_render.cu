@@ -115,6 +115,10 @@ __device__ __forceinline__ float p_rcp(float x) {
   return r;
 }
 __device__ __forceinline__ double p_rcp(double x) { return 1.0 / x; }
+// a squared distance past float32's range (a radius 1e-19 of the distance) stays
+// finite: the weight in front of it is zero
+__device__ __forceinline__ float p_finite(float x) { return fminf(x, 3.402823466e38f); }
+__device__ __forceinline__ double p_finite(double x) { return x; }
 
 // A thread's two pixels in one packed float32 value: products, sums and fmas of
 // both are one instruction (with the roundings of two), the special functions
@@ -384,6 +388,13 @@ __global__ void __launch_bounds__(PREPARE_THREADS) prepare_kernel(
     r.m11 = (T)(-sq * im.A[1] + cq * im.A[3]);
     // kA: coefficient of the position sums (dI/d rho^2 = kA g / (2 R area) with
     // g the summed weight of pixel_derivs)
+    // Far below a pixel (R < 2^-10 of one) a Gaussian's or Moffat's coefficients,
+    // F / R^3, pass float32's range while the sums behind them fall below it: a
+    // power of two (k1, exact on both sides) moves from the ones to the others.
+    const int e = sizeof(T) == 4 && !ser ? (__double2hiint(im.area * (iR * iR)) >> 20) - 1023 : 0;
+    const int up = e >= 20 ? min(2 * e, 100) : 0;
+    const double down = __hiloint2double((1023 - up) << 20, 0), back = __hiloint2double((1023 + up) << 20, 0);
+    r.k1 = (T)back;
     double kA = 0.0, amp = 0.0;
     if (ser) {
       double b = 0.0, db = 0.0;
@@ -402,14 +413,14 @@ __global__ void __launch_bounds__(PREPARE_THREADS) prepare_kernel(
       r.c4b = (T)(amp * b * LN2 * in);
       r.c5a = (T)(-kA);
     } else if (sd.type == AP_GAUSSIAN) {
-      amp = im.area * F / (2.0 * M_PI) * (iR * iR) * iq;
+      amp = im.area * F / (2.0 * M_PI) * (iR * iR) * iq * down;
       r.k0 = (T)(-0.5 * LOG2E);
       kA = -amp * iR;
       r.c4a = (T)(-2.0 * amp * iR);
       r.c4b = (T)(amp * iR);
     } else {  // Moffat
       good = good && n > 1.0;
-      amp = im.area * F * (n - 1.0) / M_PI * (iR * iR) * iq;
+      amp = im.area * F * (n - 1.0) / M_PI * (iR * iR) * iq * down;
       r.k2 = (T)n;
       kA = -2.0 * amp * n * iR;
       r.c4a = (T)(amp / (n - 1.0));
@@ -417,7 +428,7 @@ __global__ void __launch_bounds__(PREPARE_THREADS) prepare_kernel(
       r.c5a = (T)(-2.0 * amp * iR);
       r.c5b = (T)(-kA);
     }
-    r.amp = (T)amp;
+    r.amp = (T)(amp * back);
     r.c0x = (T)(-c * kA);
     r.c0y = (T)(sn * iq * kA);
     r.c1x = (T)(-sn * kA);
@@ -427,8 +438,8 @@ __global__ void __launch_bounds__(PREPARE_THREADS) prepare_kernel(
     r.c3 = (T)(kA * R * (q - iq));
     // the flux slot: the value without its factor F (area alone for Ie)
     r.c6 = (T)(ser ? im.area
-                   : sd.type == AP_GAUSSIAN ? im.area / (2.0 * M_PI) * (iR * iR) * iq
-                                            : im.area * (n - 1.0) / M_PI * (iR * iR) * iq);
+                   : down * (sd.type == AP_GAUSSIAN ? im.area / (2.0 * M_PI) * (iR * iR) * iq
+                                                    : im.area * (n - 1.0) / M_PI * (iR * iR) * iq));
   }
   if (!good) atomicCAS(status, 0, AP_ERR_NONFINITE);
   par[s] = r;
@@ -697,7 +708,7 @@ __device__ __forceinline__ void pixel_derivs(int type, const SrcPar<T>& P, int i
 #pragma unroll
   for (int bb = 0; bb < Q; ++bb) {
     const T hb = gl_hu<T>(Q, bb);
-    const T wb = gl_hw<T>(Q, bb);
+    T wb = gl_hw<T>(Q, bb);
     const T xb = x0 + P.m01 * hb, yb = y0 + P.m11 * hb;
     if (type == AP_SERSIC || type == AP_EXPONENTIAL) {
 #pragma unroll
@@ -722,11 +733,12 @@ __device__ __forceinline__ void pixel_derivs(int type, const SrcPar<T>& P, int i
         Sxy = fma(gy, x, Sxy);
       }
     } else if (type == AP_GAUSSIAN) {
+      wb *= P.k1;
 #pragma unroll
       for (int a = 0; a < Q; ++a) {
         const T ha = gl_hu<T>(Q, a);
         const T x = xb + P.m00 * ha, y = yb + P.m10 * ha;
-        const T u = fma(x, x, y * y);
+        const T u = p_finite(fma(x, x, y * y));
         const T g = (wb * gl_hw<T>(Q, a)) * p_exp2(P.k0 * u);
         S1 += g;
         Sb = fma(g, u, Sb);
@@ -737,11 +749,12 @@ __device__ __forceinline__ void pixel_derivs(int type, const SrcPar<T>& P, int i
         Sxy = fma(gy, x, Sxy);
       }
     } else {  // Moffat
+      wb *= P.k1;
 #pragma unroll
       for (int a = 0; a < Q; ++a) {
         const T ha = gl_hu<T>(Q, a);
         const T x = xb + P.m00 * ha, y = yb + P.m10 * ha;
-        const T u = fma(x, x, y * y);
+        const T u = p_finite(fma(x, x, y * y));
         const T v = (T)1 + u;
         const T lv = p_log2(v);
         const T we = (wb * gl_hw<T>(Q, a)) * p_exp2(-P.k2 * lv);
