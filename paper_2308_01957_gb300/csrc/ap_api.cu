@@ -739,10 +739,13 @@ int ap_create(ap_ctx** out, const ap_options* opt) {
   int ndev = 0;
   if (cudaGetDeviceCount(&ndev) != cudaSuccess || opt->device < 0 || opt->device >= ndev) return AP_ERR_CUDA;
   if (cudaSetDevice(opt->device) != cudaSuccess) return AP_ERR_CUDA;
+  if (upload_tables(opt->device) != 0) {
+    cudaGetLastError();
+    return AP_ERR_CUDA;
+  }
   ap_ctx* c = new ap_ctx();
   c->opt = *opt;
   c->f64 = opt->precision == AP_PREC_F64;
-  upload_gl_rule(opt->quad_order);
   bool ok = cudaEventCreateWithFlags(&c->fj.fork, cudaEventDisableTiming) == cudaSuccess;
   for (int k = 0; k < N_AUX_STREAMS && ok; ++k)
     ok = cudaStreamCreateWithFlags(&c->fj.aux[k], cudaStreamNonBlocking) == cudaSuccess &&

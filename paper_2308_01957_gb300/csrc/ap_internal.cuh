@@ -131,7 +131,7 @@ struct JcolFftWork {     // one FFT block of one free slot of one source's Jacob
 // ---------------------------------------------------------------------------
 // launchers (each TU owns its kernels; T = float or double)
 // ---------------------------------------------------------------------------
-void upload_gl_rule(int Q);  // Gauss-Legendre nodes/weights and the b_n table to device memory
+int upload_tables(int device);  // Gauss-Legendre nodes/weights and the b_n table; a cudaError_t
 
 // Let a kernel use as much dynamic shared memory as the device allows next to
 // its static shared memory (the opt-in is a cap; every launch asks for what

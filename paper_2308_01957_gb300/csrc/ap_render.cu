@@ -9,6 +9,7 @@
 #include <cmath>
 #include <vector>
 
+#include "ap_device_once.cuh"
 #include "ap_internal.cuh"
 
 namespace ap {
@@ -58,29 +59,35 @@ static void legendre_rule(int Q, double* x, double* w) {
   }
 }
 
-static void build_bn_table();
+static int upload_bn_table();
 
-void upload_gl_rule(int /*Q*/) {
-  static bool done = false;
-  if (done) return;
-  build_bn_table();
-  float hu_f[8][8] = {}, hw_f[8][8] = {};
-  double hu_d[8][8] = {}, hw_d[8][8] = {};
-  for (int Q = 1; Q <= 7; ++Q) {
-    double x[8], w[8];
-    legendre_rule(Q, x, w);
-    for (int a = 0; a < Q; ++a) {
-      hu_d[Q][a] = 0.5 * x[a];
-      hw_d[Q][a] = 0.5 * w[a];
-      hu_f[Q][a] = (float)hu_d[Q][a];
-      hw_f[Q][a] = (float)hw_d[Q][a];
+// The tables of this file on a device, before the first launch there (they are
+// uploaded once per device and process; concurrent callers wait for the upload).
+int upload_tables(int device) {
+  static DeviceOnce once;
+  return once.run(device, [] {
+    float hu_f[8][8] = {}, hw_f[8][8] = {};
+    double hu_d[8][8] = {}, hw_d[8][8] = {};
+    for (int Q = 1; Q <= 7; ++Q) {
+      double x[8], w[8];
+      legendre_rule(Q, x, w);
+      for (int a = 0; a < Q; ++a) {
+        hu_d[Q][a] = 0.5 * x[a];
+        hw_d[Q][a] = 0.5 * w[a];
+        hu_f[Q][a] = (float)hu_d[Q][a];
+        hw_f[Q][a] = (float)hw_d[Q][a];
+      }
     }
-  }
-  cudaMemcpyToSymbol(c_hu_f, hu_f, sizeof(hu_f));
-  cudaMemcpyToSymbol(c_hw_f, hw_f, sizeof(hw_f));
-  cudaMemcpyToSymbol(c_hu_d, hu_d, sizeof(hu_d));
-  cudaMemcpyToSymbol(c_hw_d, hw_d, sizeof(hw_d));
-  done = true;
+    int rc = upload_bn_table();
+    if (!rc) rc = cudaMemcpyToSymbol(c_hu_f, hu_f, sizeof(hu_f));
+    if (!rc) rc = cudaMemcpyToSymbol(c_hw_f, hw_f, sizeof(hw_f));
+    if (!rc) rc = cudaMemcpyToSymbol(c_hu_d, hu_d, sizeof(hu_d));
+    if (!rc) rc = cudaMemcpyToSymbol(c_hw_d, hw_d, sizeof(hw_d));
+    // (a copy may return before it has reached the device, which streams that do
+    // not wait for the default one would not see)
+    if (!rc) rc = cudaStreamSynchronize(cudaStreamLegacy);
+    return rc;
+  });
 }
 
 template <typename T> __device__ __forceinline__ T gl_hu(int Q, int a);
@@ -243,9 +250,9 @@ static void sersic_bn_ld(long double n, long double* b_out, long double* db_out)
   *db_out = -2.0L * (P * (std::log(b) - digamma_ld(a + 1.0L)) + b * fp / a * dS) / fp;
 }
 
-static void build_bn_table() {
+static std::vector<BnPiece> bn_table() {
   constexpr int M = BN_DEG + 1;
-  static BnPiece tab[BN_PIECES];
+  std::vector<BnPiece> tab(BN_PIECES);
   const long double pi = 3.14159265358979323846264338327950288L;
   for (int p = 0; p < BN_PIECES; ++p) {
     const long double n0 = BN_MIN * std::exp2(0.25L * p), n1 = n0 * std::exp2(0.25L);
@@ -283,7 +290,12 @@ static void build_bn_table() {
       tab[p].db[k] = (double)pw[1][BN_DEG - k];
     }
   }
-  cudaMemcpyToSymbol(c_bn, tab, sizeof(tab));
+  return tab;
+}
+
+static int upload_bn_table() {
+  static const std::vector<BnPiece> tab = bn_table();   // once per process
+  return cudaMemcpyToSymbol(c_bn, tab.data(), tab.size() * sizeof(BnPiece));
 }
 
 // b_n and db/dn for n in [BN_MIN, BN_MAX]
