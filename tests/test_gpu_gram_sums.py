@@ -1,8 +1,10 @@
-"""The sums of J^T W J over tiles past float32's range."""
+"""The sums of J^T W J over tiles: past float32's range, and at the sizes where
+their form changes (pairs of up to 2048 values, runs of up to 8192 values, tiles of
+up to 22 sources)."""
 import numpy as np
 import pytest
 
-from _helpers import O, TOL_GRAD, device_context
+from _helpers import O, TOL_GRAD, configs, device_context, with_data
 from synthetic.problem import ImageSpec, Problem, SourceSpec
 
 torch = pytest.importorskip("torch")
@@ -26,6 +28,19 @@ def _source(type_, image, win, pidx, pfix=()):
     i[:len(pidx)] = pidx
     f[:len(pfix)] = pfix
     return SourceSpec(type_, image, win, False, i, f)
+
+
+def _check_jtwj(pr, tol=TOL_GRAD, **options):
+    from paper_2308_01957_gb300 import api
+    ctx = api.Context("mixed", pr.quad_order, device=0, **options)
+    ctx.set_problem(api.to_device_images(pr.images), pr.sources, pr.n_params)
+    ref, _ = O.normal_equations(pr, pr.theta_init)
+    _, csr = ctx.normal_eq(pr.theta_init)
+    JtWJ = ctx.jtwj_dense(csr)
+    d = np.sqrt(np.maximum(np.diag(ref), 1e-300))
+    assert (np.abs(JtWJ - ref) / np.outer(d, d)).max() <= tol
+    assert ctx.status() == 0
+    return csr
 
 
 @pytest.mark.parametrize("h,w", [(64, 64), (736, 736), (48, 43696)])
@@ -54,3 +69,43 @@ def test_entries_past_float32_range(h, w):
     want = np.linalg.solve(got + 1e-3 * np.diag(np.diag(got)), _np(jtwr))
     np.testing.assert_allclose(_np(delta), want, rtol=1e-10)
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("n_tiles", [227, 228, 910, 911, 1821])
+@pytest.mark.parametrize("shared", [False, True])
+def test_pair_sums_at_run_boundaries(n_tiles, shared):
+    """A strip of n 16 x 16 tiles under a plane sky (9 values per tile: 2043 and
+    2052 values on both sides of a warp's 2048; 910 tiles fill a run of 8192
+    values, 911 start a second, 1821 a third) and a star; shared: two such strips
+    with the same parameters, whose pairs add to the same entries."""
+    h, w = 16, 16 * n_tiles
+    rng = np.random.default_rng(n_tiles)
+    images, sources = [], []
+    for k in range(2 if shared else 1):
+        images.append(ImageSpec(h, w, np.eye(2), np.array([-0.5 * w, -8.0]),
+                                data=rng.standard_normal((h, w)).astype(np.float32),
+                                variance=rng.uniform(0.5, 1.5, (h, w)).astype(np.float32)))
+        sources.append(_source(O.SKY_PLANE, k, (0, w, 0, h), [0, 1, 2]))
+        sources.append(_source(O.GAUSSIAN, k, (3, 40, 0, h), [3, 4, -1, -1, -1, 5], [0.0, 0.0, 0.7, 0.4, 2.5, 0.0]))
+    theta = np.array([1.0, 1e-3, -2e-3, -0.5 * w + 20.4, 0.7, 50.0])
+    _check_jtwj(Problem("strip", images, sources, 6, theta, theta))
+
+
+@pytest.mark.parametrize("nm", [20, 21])
+def test_tiles_at_the_staged_pair_limit(nm):
+    """A tile of 22 sources (253 pairs, offsets kept in shared memory) and one of 23 (276, read in place)."""
+    pr = with_data(configs.crowded_field(f"pairs_{nm}", configs.SEED_BASE + 97, 16, 16, 1, nm, configs.psf_moffat(5, 2.5)))
+    assert len(pr.sources) == nm + 2
+    _check_jtwj(pr)
+
+
+def test_gram_tc_min_changes_nothing():
+    """The option is still accepted (a negative one refused): the same entries bit by bit."""
+    from paper_2308_01957_gb300 import api
+    from paper_2308_01957_gb300._lib import ApError
+    pr = with_data(configs.crowded_field("graded_tiles", configs.SEED_BASE + 72, 96, 160, 12, 20,
+                                         configs.psf_moffat(5, 2.5)))
+    vals = [_check_jtwj(pr, jcol="direct", conv_variant=1, gram_tc_min=m)[2] for m in (0, 1, 257)]
+    assert torch.equal(vals[0], vals[1]) and torch.equal(vals[0], vals[2])
+    with pytest.raises(ApError):
+        api.Context("mixed", pr.quad_order, device=0, gram_tc_min=-1)
