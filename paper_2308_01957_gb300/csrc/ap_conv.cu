@@ -441,7 +441,7 @@ static int configure_one(int Kmax) {
     CALL(0, __VA_ARGS__);                                                         \
   }
 
-// only the two fast tile shapes get NC instantiations; the others run generic
+// only the three shapes of 16 x 8 threads get NC instantiations; the others run generic
 __host__ __device__ constexpr bool fast_shape(int bx, int by, int ry) {
   return bx == 16 && by == 8 && (ry == 2 || ry == 4 || ry == 8);
 }

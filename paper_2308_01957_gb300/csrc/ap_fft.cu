@@ -203,7 +203,10 @@ __device__ __forceinline__ void fft_lines(float2* a, int nlines, const float2* t
 // passes through shared memory and four barriers less than a forward and an
 // inverse transform one after the other: with the weights of the outputs loaded
 // eight rows at a time, 21.5 -> 19.6 ms for the joint fit's columns, 2.59 -> 2.42 ms
-// for a 1536^2 field with a 51 x 51 PSF.  (Whole lines in the registers of one or
+// for a 1536^2 field with a 51 x 51 PSF.  (Of the 21.5 some 2 ms came with the
+// sqrt(w)-scaled tile blocks that the columns are stored in for J^T W J; stored row
+// by row and unscaled they took 17.8 ms in the benchmark's joint fit, now 18.1.)
+// (Whole lines in the registers of one or
 // two threads, eight passes through shared memory instead of sixteen, left too
 // few warps to hide the loads: 35 ms.)
 template <int LEN, int NT, int ES, int LS, class LD, class MUL>

@@ -24,9 +24,12 @@
 // the same registers.  The four warps' 64-pixel float32 sums are joined by
 // compensated additions and kept as an unevaluated pair hi + lo of floats
 // (float64 conversions and additions for every entry of every tile would
-// occupy the thin float64 pipe longer than the MMAs take).  Bound by the
-// warp-MMA rate (a 48-column tile: 1152 MMAs, 2300 clocks of an SM at the
-// measured 303 TFLOP/s).  tcgen05 does not pay at these shapes: its M = 128 by
+// occupy the thin float64 pipe longer than the MMAs take); the pair keeps about 48
+// bits of sums of float32 products.  A 48-column tile is 1152 MMAs, 2300 clocks of an
+// SM at the measured 303 TFLOP/s; the kernel takes some three times that (tensor
+// pipe 27 to 31 % busy on the two largest forms), because a CTA loads, multiplies
+// and writes one tile after the other and two to six CTAs an SM, as many as the
+// registers allow, do not cover it.  tcgen05 does not pay at these shapes: its M = 128 by
 // N = C MMA reads 4 + C/32 KB of operands from shared memory for
 // 128 x C x 8 products, so a 48-column tile takes some 1400 clocks of
 // shared-memory bandwidth for the MMAs and 1150 more to split and store both
@@ -249,8 +252,8 @@ __global__ void __launch_bounds__(GT_THREADS, (gt_min_ctas<NM, NN, DIAG>())) gra
     if (ph == 0 && staged)
       for (int p = tid; p < L * (L + 1) / 2; p += GT_THREADS) s_tab[p] = tab[p];
     if (!__syncthreads_and(mbar_wait(mbar, ph & 1))) {
-      // the copies did not arrive within the limit: one more wait, so that
-      // none is in flight when the CTA leaves
+      // the copies did not arrive within the limit: an error, and one more
+      // wait of the same length for those still in flight before the CTA leaves
       if (tid == 0) atomicCAS(status, 0, AP_ERR_TIMEOUT);
       mbar_wait(mbar, ph & 1);
       return;
@@ -596,7 +599,7 @@ __global__ void __launch_bounds__(256) gram_reduce_kernel(const GramPair* __rest
   }
 }
 
-// the other pairs: a CTA per run of up to GRAM_RUN_TILES tiles; the CTA that
+// the other pairs: a CTA per run of some GRAM_RUN_VALUES values; the CTA that
 // finishes a pair last adds its runs in order
 template <typename V>
 __global__ void __launch_bounds__(256) gram_reduce_run_kernel(const GramPair* __restrict__ pairs,

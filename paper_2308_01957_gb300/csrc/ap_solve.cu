@@ -74,8 +74,8 @@ __device__ __forceinline__ double block_max(double v, double* red) {
 // Cholesky in the form L diag(d) L^T (the same pivots, no square roots), right
 // looking, one barrier per column: a thread owns a row (two threads share its
 // columns) and updates it with the column's unscaled entries; the scaled ones go to
-// the upper triangle; the thread that completes the next pivot also takes its
-// reciprocal (in every thread, the divisions would take as long as the updates).
+// the upper triangle; the thread that completes the next pivot also divides one by
+// it (in every thread, the divisions would take as long as the updates).
 // The right-hand side rides along as row n, which makes the forward substitution
 // part of the factorisation; one warp does the back substitution by columns.
 // Bound by the float64 pipe (a warp's FMA holds it for some 17 clocks, n^3 / 170
