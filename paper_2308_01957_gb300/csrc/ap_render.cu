@@ -124,8 +124,12 @@ __device__ __forceinline__ float p_rcp(float x) {
 }
 __device__ __forceinline__ double p_rcp(double x) { return 1.0 / x; }
 // a squared distance past float32's range (a radius 1e-19 of the distance) stays
-// finite: the weight in front of it is zero
-__device__ __forceinline__ float p_finite(float x) { return fminf(x, 3.402823466e38f); }
+// finite: the weight in front of it is zero; NaN stays NaN
+__device__ __forceinline__ float p_finite(float x) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(x), "f"(3.402823466e38f));
+  return r;
+}
 __device__ __forceinline__ double p_finite(double x) { return x; }
 
 // A thread's two pixels in one packed float32 value: products, sums and fmas of

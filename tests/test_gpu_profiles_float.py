@@ -148,3 +148,18 @@ def test_gradient_of_the_wings_of_a_tiny_moffat(R):
     _, g = ctx.eval(theta)
     assert_grad_close(_np(g), O.gradient(pr, theta), grad_scale(pr, theta), TOL_GRAD)
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("type_", [O.GAUSSIAN, O.MOFFAT])
+def test_a_position_that_is_no_number_stays_one(type_):
+    """A fixed centre that is NaN reaches every entry of a free radius and flux, and the status word."""
+    from paper_2308_01957_gb300 import _lib
+    slots = [math.nan, Y0, Q, PA, 2.0, 100.0] if type_ == O.GAUSSIAN else [math.nan, Y0, Q, PA, 2.5, 2.0, 100.0]
+    pr = _problem(type_, slots, h=24, w=24, free=(len(slots) - 2, len(slots) - 1), sky=1.0)
+    pr.images[0].data = np.ones((24, 24), dtype=np.float32)
+    pr.images[0].variance = np.ones((24, 24), dtype=np.float32)
+    ctx = device_context(pr, "mixed")
+    _, csr = ctx.normal_eq(pr.theta_init)
+    M = ctx.jtwj_dense(csr)
+    assert np.isnan(M[:2, :2]).all() and np.isfinite(M[2, 2]), M
+    assert ctx.status() == _lib.AP_ERR_NONFINITE
